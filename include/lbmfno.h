@@ -104,7 +104,8 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
 
 /* Advance every grid by nsteps fused collide+stream steps (Sec. 2.1 loop:
  * equilibrium, SRT collision, streaming with halfway bounce-back, moments).
- * One kernel launch per step. */
+ * One kernel launch per two steps (a pass over the populations that takes both), and
+ * one for a last odd step; bitwise equal to single steps. */
 int lbm_step(lbm_handle* h, int nsteps, void* stream);
 
 /*

@@ -42,7 +42,7 @@ def _deps_mtime() -> float:
 # Per-file flags.  The LBM step kernel exists in several compiled variants (tile shapes,
 # modes) that must round identically; without automatic multiply-add contraction the
 # rounding of every expression is fixed by the source (fused operations are explicit fmaf).
-FILE_FLAGS = {"lbm.cu": ["-fmad=false"]}
+FILE_FLAGS = {"lbm.cu": ["-fmad=false"], "lbm_sweep.cu": ["-fmad=false"]}
 
 
 def _compile(src: str, extra) -> str:

@@ -820,7 +820,7 @@ __global__ void __launch_bounds__(kBlock) k_vorticity(const GridDev* __restrict_
 // ------------------------------------------------------------ host side ---
 struct WsPlan {
   size_t grids_off, uprev_off, seg_off, partial_off, stats_off, status_off, bar_off, tiles_off,
-      total;
+      sweep_off, total;
 };
 
 // Scratch of one statistics evaluation: FP32 row-segment partials, FP64 block sums,
@@ -842,7 +842,7 @@ static int plan_layout(const lbm_grid* grids, int ngrids, lbm_layout* lay,
   LBM_REQUIRE(grids != nullptr && ngrids > 0, "lbm: need at least one grid");
   size_t f = 0, words = 0, cells = 0;
   long long blk = 0, tiles = 0, rblk = 0;
-  if (gd) gd->clear();
+  std::vector<GridDev> all;
   // Population-major batch layout: plane i holds population i of every grid, grid after
   // grid (each grid ny rows of pitch floats), so a batch of small grids streams nine
   // contiguous planes exactly like one tall grid.
@@ -907,8 +907,9 @@ static int plan_layout(const lbm_grid* grids, int ngrids, lbm_layout* lay,
     rblk += d.nrblk;
     LBM_REQUIRE(blk < (1LL << 30) && tiles < (1LL << 30),
                 "lbm: batch too large");
-    if (gd) gd->push_back(d);
+    all.push_back(d);
   }
+  if (gd) *gd = all;
   WsPlan w{};
   w.grids_off = 0;
   w.uprev_off = align_up(sizeof(GridDev) * ngrids, 256);
@@ -924,7 +925,10 @@ static int plan_layout(const lbm_grid* grids, int ngrids, lbm_layout* lay,
     for (int k = 0; k < ngrids; ++k)
       tiles_all += (size_t)((grids[k].nx + kSeg - 1) / kSeg) *
                    ((grids[k].ny + kStepVariants[v].ty - 1) / kStepVariants[v].ty);
-  w.total = align_up(w.tiles_off + tiles_all * sizeof(int4), 256);
+  w.sweep_off = align_up(w.tiles_off + tiles_all * sizeof(int4), 256);
+  std::vector<SweepTask> sweep;
+  sweep_plan(all, &sweep);
+  w.total = align_up(w.sweep_off + sweep.size() * sizeof(SweepTask), 256);
   lay->f_elems = (size_t)kQ * plane_all;
   lay->mask_words = words;
   lay->cells = cells;
@@ -1114,6 +1118,10 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
   }
   for (int v = 0; v < LBM_STEP_VARIANTS; ++v)
     h->tiles_d[v] = reinterpret_cast<int4*>(ws + wp.tiles_off) + tiles_at[v];
+  std::vector<SweepTask> sweep;
+  sweep_plan(h->gd, &sweep);
+  h->sweep_d = reinterpret_cast<SweepTask*>(ws + wp.sweep_off);
+  h->sweep_ctas = (int)(sweep.size() / kSweepWarps);
   h->stats_h.assign((size_t)ngrids * R_COUNT, 0.0);
   h->u_max2 = (float)(u_max * u_max);
   cudaStream_t s = S(stream);
@@ -1133,7 +1141,7 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
                                                            sv.smem_of(m)) == cudaSuccess;
       h->blocks_per_sm_v[v] = h->blocks_per_sm_vm[v][kModeStep];
     }
-    if (ok) ok = reinit_init(h) == LBM_OK;
+    if (ok) ok = reinit_init(h) == LBM_OK && sweep_init() == LBM_OK;
     if (!ok) {
       set_error("lbm_init: %s", cudaGetErrorString(cudaGetLastError()));
       delete h;
@@ -1153,6 +1161,8 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
       cudaMemsetAsync(h->status_d, 0, sizeof(unsigned), s) != cudaSuccess ||
       cudaMemcpyAsync(h->tiles_d[0], tiles.data(), tiles.size() * sizeof(int4),
                       cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      cudaMemcpyAsync(h->sweep_d, sweep.data(), sweep.size() * sizeof(SweepTask),
+                      cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("lbm_init: %s", cudaGetErrorString(cudaGetLastError()));
     return fail(LBM_ERR_CUDA);
@@ -1171,7 +1181,12 @@ int lbm_step(lbm_handle* h, int nsteps, void* stream) {
     h->steps += nsteps;
     return LBM_OK;
   }
-  for (int k = 0; k < nsteps; ++k) {
+  int left = nsteps;
+  for (; left >= kSweepSteps; left -= kSweepSteps) {
+    LBM_TRY(sweep_launch(h, h->f[h->cur], h->f[h->cur ^ 1], s));
+    h->cur ^= 1;
+  }
+  for (; left > 0; --left) {
     LBM_TRY(launch_step(h, h->variant, kModeStep, h->f[h->cur], h->f[h->cur ^ 1], s));
     h->cur ^= 1;
   }

@@ -4,6 +4,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "lbm_sweep.cuh"
 
 namespace lbmfno {
 
@@ -22,6 +23,8 @@ struct Handle {
   bool persistent = false;     // lbm_step runs nsteps > 1 in one multi-step launch
   unsigned* bar_count = nullptr;  // grid-barrier counter of the multi-step launch
   int4* tiles_d[LBM_STEP_VARIANTS] = {};      // per-shape tile descriptors (workspace)
+  struct SweepTask* sweep_d = nullptr;  // tasks of a multi-step pass (workspace)
+  int sweep_ctas = 0;
   unsigned* status_d = nullptr;
   unsigned status_h = 0;
   const uint32_t* mask = nullptr;
