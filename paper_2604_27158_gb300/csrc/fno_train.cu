@@ -31,13 +31,17 @@ namespace {
 
 inline cudaStream_t TS(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-constexpr int kPwPix = 128;      // pixels per block of the pointwise kernel
-constexpr int kWgThreads = 256;  // threads of the weight-gradient kernel
-constexpr int kWgPairs = 17;     // (o, i) pairs per thread: 64 x (64 + 1) <= 256 * 17
-constexpr int kWgTile = 32;      // pixels staged per iteration
-constexpr int kSpecThreads = 256;
-constexpr int kAccMax = 16;      // spectral accumulators per thread
 constexpr int kTrModesMax = 32;
+constexpr int kTrSms = 152;
+constexpr int kPwThreads = 256;  // threads of the pointwise kernel
+constexpr int kPwCtas = 3;       // its blocks a multiprocessor (shared memory, registers)
+constexpr int kWgThreads = 256;  // threads of the weight-gradient kernel
+constexpr int kWgTile = 64;      // pixels of one of its stages
+constexpr int kDftM = 128;       // (row, channel) pairs of an x-DFT block
+constexpr int kDftX = 32;        // columns of one of its stages
+constexpr int kDftYA = 8;        // kept rows of a forward y-DFT thread
+constexpr int kDftYC = 64;       // rows of one of its stages
+constexpr int kInvY = 8;         // rows of an inverse y-DFT thread
 
 struct TrOff {
   size_t lift0_w, lift0_b, lift1_w, lift1_b;
@@ -94,8 +98,9 @@ struct TrPlan {
   // saved, in floats
   size_t xin, h1pre, theta, zpre, xh, hdpre, saved_floats;
   // workspace, in bytes
-  size_t rt, x1, yh, dyh, z, s, ta, tb, dz, part, twx, twy, ycl, ws_bytes;
+  size_t rt, x1, yh, dyh, z, ta, tb, part, ex, ey, ycl, ws_bytes;
   int wg_blocks;
+  int np, ng, ep;  // x-DFT: kx pairs a thread, thread groups, floats a row of the table
 };
 
 TrPlan tr_plan(const fno_config& c, int B, int H, int W) {
@@ -133,14 +138,20 @@ TrPlan tr_plan(const fno_config& c, int B, int H, int W) {
   t.yh = take(spec * sizeof(float2));
   t.dyh = take(spec * sizeof(float2));
   t.z = take((size_t)B * H * m * C * sizeof(float2));
-  t.s = take(P * C * sizeof(float));
   t.ta = take(P * wide * sizeof(float));
   t.tb = take(P * wide * sizeof(float));
-  t.dz = take(P * wide * sizeof(float));
-  t.wg_blocks = (int)std::min<size_t>(1024, (P + 511) / 512);
+  t.wg_blocks = (int)std::min<size_t>(2 * kTrSms, (P + 4 * kWgTile - 1) / (4 * kWgTile));
   t.part = take((size_t)t.wg_blocks * 64 * 65 * sizeof(float));
-  t.twx = take((size_t)W * sizeof(float2));
-  t.twy = take((size_t)H * sizeof(float2));
+  // kx pairs a thread of the x-DFT: the split with the fewest padded pairs
+  t.np = 4;
+  for (int np : {6, 7, 8})
+    if ((m + np - 1) / np * np < (m + t.np - 1) / t.np * t.np ||
+        ((m + np - 1) / np * np == (m + t.np - 1) / t.np * t.np && np > t.np))
+      t.np = np;
+  t.ng = (int)((m + t.np - 1) / t.np);
+  t.ep = (2 * t.np * t.ng + 3) / 4 * 4;
+  t.ex = take((size_t)W * t.ep * sizeof(float));
+  t.ey = take((size_t)H * 2 * m * sizeof(float4));
   t.ycl = take(P * c.c_out * sizeof(float));
   t.ws_bytes = b;
   return t;
@@ -161,13 +172,26 @@ __device__ __forceinline__ float bf16r(float v) {
   return __bfloat162float(__float2bfloat16_rn(v));
 }
 
-__global__ void k_tr_twiddle(float2* __restrict__ tw, int N) {
+// ex[x][2 kx] = (cos, -sin)(2 pi kx x / W), 0 for kx >= m.
+__global__ void k_tr_ex(float* __restrict__ ex, int W, int m, int ep) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < N) {
-    double s, c;
-    sincospi(2.0 * (double)t / (double)N, &s, &c);
-    tw[t] = make_float2((float)c, (float)s);
-  }
+  if (t >= W * (ep / 2)) return;
+  const int x = t / (ep / 2), kx = t - x * (ep / 2);
+  double s = 0.0, c = 0.0;
+  if (kx < m) sincospi(2.0 * (double)((long long)kx * x % W) / (double)W, &s, &c);
+  ex[x * ep + 2 * kx] = (float)c;
+  ex[x * ep + 2 * kx + 1] = (float)-s;
+}
+// ey[y][a] = (cos, -sin, sin, cos)(2 pi ky(a) y / H), ky(a) = a (a < m) or H - 2m + a: a
+// complex product with e^{-i phi} is two packed multiply-adds.
+__global__ void k_tr_ey(float4* __restrict__ ey, int H, int m) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= H * 2 * m) return;
+  const int y = t / (2 * m), a = t - y * (2 * m);
+  const int ky = a < m ? a : H - 2 * m + a;
+  double s, c;
+  sincospi(2.0 * (double)((long long)ky * y % H) / (double)H, &s, &c);
+  ey[t] = make_float4((float)c, (float)-s, (float)s, (float)c);
 }
 
 // Rt[layer][mode][i][o] = R[i][o][ky][kx] (mode = a m + kx; a < m: r1 at ky = a,
@@ -212,235 +236,520 @@ __global__ void k_tr_xin(const float* __restrict__ in, float* __restrict__ xin, 
   xin[p * cin2 + cin + 1] = bf16r((float)y / (float)max(H - 1, 1));
 }
 
-// Pointwise linear layer over kPwPix pixels per block:
-//   v[p][o] = add[p][o] + bias[o] + sum_i Wm(o, i) * A(in[p][i]),
+__device__ __forceinline__ void cpa16(float* s, const float* g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(s)),
+               "l"(g)
+               : "memory");
+}
+__device__ __forceinline__ void cpa8(float* s, const float* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(s)),
+               "l"(g)
+               : "memory");
+}
+__device__ __forceinline__ void cpa4(float* s, const float* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(s)),
+               "l"(g)
+               : "memory");
+}
+__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cpa_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+
+// Pointwise linear layer, with the inverse x-DFT of a row's coefficients added:
+//   v[p][o] = bias[o] + sum_i Wm(o, i) A(in[p][i]) + sum_kx Re(z[row][kx][o] e^{+2 pi i kx x / W}),
 //   Wm(o, i) = trans ? w[i * cout + o] : w[o * cin + i],  A = sigma if in_act else identity;
-//   pre[p][o] = v (if pre != null);  out[p][o] = out_act ? sigma(v) : v.
-__global__ void __launch_bounds__(kPwPix) k_tr_pw(const float* __restrict__ in, int cin,
-                                                  const float* __restrict__ w, int trans,
-                                                  const float* __restrict__ bias,
-                                                  const float* __restrict__ add, int cout,
-                                                  float* __restrict__ pre, float* __restrict__ out,
-                                                  int in_act, int out_act, int act, size_t P) {
-  extern __shared__ float sm[];
-  float* ws = sm;                               // [cout][cin]
-  float* is = ws + cout * cin;                  // [kPwPix][cin + 1]
-  float* os = is + kPwPix * (cin + 1);          // [kPwPix][cout + 1]
-  const size_t p0 = (size_t)blockIdx.x * kPwPix;
-  const int np = (int)min((size_t)kPwPix, P - p0);
-  for (int j = threadIdx.x; j < cout * cin; j += kPwPix) {
-    const int o = j / cin, i = j - o * cin;
-    ws[j] = trans ? w[(size_t)i * cout + o] : w[j];
-  }
-  for (int j = threadIdx.x; j < np * cin; j += kPwPix) {
-    const int t = j / cin, i = j - t * cin;
-    const float v = in[p0 * cin + j];
-    is[t * (cin + 1) + i] = in_act ? tr_act(v, act) : v;
-  }
-  for (int j = threadIdx.x; j < np * cout; j += kPwPix) {
-    const int t = j / cout, o = j - t * cout;
-    os[t * (cout + 1) + o] = (add ? add[p0 * cout + j] : 0.0f) + (bias ? bias[o] : 0.0f);
-  }
+//   pre[p][o] = v (if pre);  out[p][o] = sigma(v) if out_act, v * sigma'(dz[p][o]) if dz, else v
+// (planar: out is [b][cout][hw]).  One contraction over cin + 2m terms: the columns of A are
+// the inputs and the (cos, -sin) table of the pixel's column, those of B the weights and the
+// row's coefficients (Re, Im).
+//
+// FP32 multiply-adds bound it (64 channels, 13 modes: 92 terms an output against 16 bytes).  A
+// thread owns PPT pixels x 4 outputs and packs its accumulators over pairs of terms, so both
+// operands are plain 16-byte shared loads of four terms; row pitches are an odd number of
+// 16-byte units (no bank conflicts) and weights are stored with the rows of the four outputs
+// of a thread G apart.  A block walks a contiguous range of tiles; the next tile (and row's
+// coefficients) is copied while the current one is summed.
+struct PwArgs {
+  const float* in;
+  const float* w;
+  const float* bias;
+  const float2* z;   // [row][m][cout], or null
+  const float* ex;
+  const float* dz;
+  float* pre;
+  float* out;
+  size_t P, hw;
+  int cin, cout, trans, in_act, out_act, act, planar;
+  int W, m, ep;      // row length; modes and table pitch (z)
+  int ap, wp, zp;    // row pitches: inputs, weights, coefficients
+  int ntiles, tpr;   // tiles; tiles a row (z)
+};
+template <int OP, int PT>
+__global__ void __launch_bounds__(kPwThreads, kPwCtas) k_tr_pw(const PwArgs a) {
+  constexpr int G = OP / 4, NPG = kPwThreads / G, PPT = PT / NPG;
+  static_assert(PPT >= 1 && NPG * PPT == PT, "pixels a thread");
+  extern __shared__ __align__(16) float sm[];
+  float* As = sm;                       // [2][PT][ap]: inputs, then the table's columns
+  float* Ws = As + 2 * PT * a.ap;       // [OP][wp], output o in row (o % 4) * G + o / 4
+  float* Zs = Ws + OP * a.wp;           // [2][OP][zp], rows as Ws
+  const int ap = a.ap, wp = a.wp, zp = a.zp, cin = a.cin, cout = a.cout;
+  const int cin4 = (cin + 3) & ~3, m2 = a.z ? 2 * a.m : 0, m24 = (m2 + 3) & ~3;
+  for (int j = threadIdx.x; j < 2 * PT * ap + OP * (wp + 2 * zp); j += kPwThreads) sm[j] = 0.0f;
   __syncthreads();
-  const int t = threadIdx.x;
-  if (t < np) {
-    const float* ir = is + t * (cin + 1);
-    float* orow = os + t * (cout + 1);
-    for (int o = 0; o < cout; ++o) {
-      const float* wr = ws + o * cin;
-      float acc = 0.0f;
-      for (int i = 0; i < cin; ++i) acc = fmaf(wr[i], ir[i], acc);
-      orow[o] += acc;
-    }
+  for (int j = threadIdx.x; j < cout * cin; j += kPwThreads) {
+    const int o = a.trans ? j % cout : j / cin, i = a.trans ? j / cout : j - o * cin;
+    Ws[((o & 3) * G + (o >> 2)) * wp + i] = a.w[j];
   }
-  __syncthreads();
-  for (int j = threadIdx.x; j < np * cout; j += kPwPix) {
-    const int tt = j / cout, o = j - tt * cout;
-    const float v = os[tt * (cout + 1) + o];
-    if (pre) pre[p0 * cout + j] = v;
-    out[p0 * cout + j] = out_act ? tr_act(v, act) : v;
-  }
-}
-
-// dz = g * sigma'(z), elementwise
-__global__ void k_tr_act_bwd(const float* __restrict__ g, const float* __restrict__ z,
-                             float* __restrict__ dz, size_t n, int act) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    dz[i] = g[i] * tr_dact(z[i], act);
-}
-
-// Block partials of dW[o][i] = sum_p dz[p][o] A(in[p][i]) and db[o] = sum_p dz[p][o]
-// (pair (o, cin) of the partial is db).  Block k covers a contiguous pixel range.
-__global__ void __launch_bounds__(kWgThreads) k_tr_wgrad(const float* __restrict__ dz, int cout,
-                                                         const float* __restrict__ in, int cin,
-                                                         int in_act, int act, size_t P,
-                                                         float* __restrict__ part) {
-  __shared__ float ds[kWgTile][65];
-  __shared__ float is[kWgTile][66];
-  const int npairs = cout * (cin + 1);
-  const size_t per = (P + gridDim.x - 1) / gridDim.x;
-  const size_t pa = (size_t)blockIdx.x * per;
-  const size_t pb = min(P, pa + per);
-  float acc[kWgPairs];
+  const int og = threadIdx.x % G, pg = threadIdx.x / G;
+  float bias[4];
 #pragma unroll
-  for (int k = 0; k < kWgPairs; ++k) acc[k] = 0.0f;
-  for (size_t q0 = pa; q0 < pb; q0 += kWgTile) {
-    const int nt = (int)min((size_t)kWgTile, pb - q0);
-    __syncthreads();
-    for (int j = threadIdx.x; j < kWgTile * cout; j += kWgThreads) {
-      const int t = j / cout, o = j - t * cout;
-      ds[t][o] = t < nt ? dz[(q0 + t) * cout + o] : 0.0f;
+  for (int j = 0; j < 4; ++j) bias[j] = a.bias && og * 4 + j < cout ? a.bias[og * 4 + j] : 0.0f;
+  const int t0 = (int)((long long)a.ntiles * blockIdx.x / gridDim.x);
+  const int t1 = (int)((long long)a.ntiles * (blockIdx.x + 1) / gridDim.x);
+  // first pixel and pixels of tile t (x0: its column, z)
+  auto place = [&](int t, size_t& p0, int& np, int& x0) {
+    if (m2) {
+      const int row = t / a.tpr;
+      x0 = (t - row * a.tpr) * PT;
+      p0 = (size_t)row * a.W + x0;
+      np = min(PT, a.W - x0);
+    } else {
+      x0 = 0;
+      p0 = (size_t)t * PT;
+      np = (int)min((size_t)PT, a.P - p0);
     }
-    for (int j = threadIdx.x; j < kWgTile * (cin + 1); j += kWgThreads) {
-      const int t = j / (cin + 1), i = j - t * (cin + 1);
-      float v = 0.0f;
-      if (t < nt) {
-        if (i == cin) {
-          v = 1.0f;
-        } else {
-          v = in[(q0 + t) * cin + i];
-          if (in_act) v = tr_act(v, act);
+  };
+  auto load = [&](int t, int buf, bool zrow) {
+    size_t p0;
+    int np, x0;
+    place(t, p0, np, x0);
+    float* A = As + buf * PT * ap;
+    const float* src = a.in + p0 * cin;
+    if ((cin & 3) == 0) {
+      const int q = cin >> 2;
+      for (int j = threadIdx.x; j < np * q; j += kPwThreads) {
+        const int p = j / q;
+        cpa16(A + p * ap + 4 * (j - p * q), src + 4 * j);
+      }
+    } else {
+      for (int j = threadIdx.x; j < np * cin; j += kPwThreads) {
+        const int p = j / cin;
+        cpa4(A + p * ap + (j - p * cin), src + j);
+      }
+    }
+    if (m2) {
+      for (int j = threadIdx.x; j < np * a.m; j += kPwThreads) {
+        const int p = j / a.m, c = j - p * a.m;
+        cpa8(A + p * ap + cin4 + 2 * c, a.ex + (size_t)(x0 + p) * a.ep + 2 * c);
+      }
+      if (zrow) {
+        const int row = t / a.tpr;
+        float* Z = Zs + (row & 1) * OP * zp;
+        const float* zr = reinterpret_cast<const float*>(a.z + (size_t)row * a.m * cout);
+        for (int j = threadIdx.x; j < a.m * cout; j += kPwThreads) {
+          const int kx = j / cout, o = j - kx * cout;
+          cpa8(Z + ((o & 3) * G + (o >> 2)) * zp + 2 * kx, zr + 2 * j);
         }
       }
-      is[t][i] = v;
     }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kWgPairs; ++k) {
-      const int pr = threadIdx.x + k * kWgThreads;
-      if (pr < npairs) {
-        const int o = pr / (cin + 1), i = pr - o * (cin + 1);
-        float a = acc[k];
-        for (int t = 0; t < kWgTile; ++t) a = fmaf(ds[t][o], is[t][i], a);
-        acc[k] = a;
+  };
+  if (t0 < t1) load(t0, 0, true);
+  cpa_commit();
+  for (int t = t0; t < t1; ++t) {
+    const int buf = (t - t0) & 1;
+    size_t p0;
+    int np, x0;
+    place(t, p0, np, x0);
+    if (t + 1 < t1) load(t + 1, buf ^ 1, m2 && (t + 1) % a.tpr == 0);
+    cpa_commit();
+    cpa_wait<1>();
+    float* A = As + buf * PT * ap;
+    if (a.in_act) {  // each thread the elements it copied
+      if ((cin & 3) == 0) {
+        const int q = cin >> 2;
+        for (int j = threadIdx.x; j < np * q; j += kPwThreads) {
+          const int p = j / q;
+          float4* e = reinterpret_cast<float4*>(A + p * ap + 4 * (j - p * q));
+          const float4 v = *e;
+          *e = make_float4(tr_act(v.x, a.act), tr_act(v.y, a.act), tr_act(v.z, a.act),
+                           tr_act(v.w, a.act));
+        }
+      } else {
+        for (int j = threadIdx.x; j < np * cin; j += kPwThreads) {
+          const int p = j / cin;
+          float* e = A + p * ap + (j - p * cin);
+          *e = tr_act(*e, a.act);
+        }
       }
     }
-  }
-#pragma unroll
-  for (int k = 0; k < kWgPairs; ++k) {
-    const int pr = threadIdx.x + k * kWgThreads;
-    if (pr < npairs) part[(size_t)blockIdx.x * npairs + pr] = acc[k];
-  }
-}
-
-// Ordered sum of the block partials into dW (cout x cin) and db (cout).
-__global__ void k_tr_wgrad_reduce(const float* __restrict__ part, int nblk, int cout, int cin,
-                                  float* __restrict__ dw, float* __restrict__ db) {
-  const int npairs = cout * (cin + 1);
-  const int pr = blockIdx.x * blockDim.x + threadIdx.x;
-  if (pr >= npairs) return;
-  float s = 0.0f;
-  for (int k = 0; k < nblk; ++k) s += part[(size_t)k * npairs + pr];
-  const int o = pr / (cin + 1), i = pr - o * (cin + 1);
-  if (i == cin)
-    db[o] = s;
-  else
-    dw[o * cin + i] = s;
-}
-
-// Forward x-DFT of each row: X1[row][kx][c] = sum_x f[row][x][c] e^{-2 pi i kx x / W}.
-__global__ void __launch_bounds__(kSpecThreads) k_tr_dft_x(const float* __restrict__ f,
-                                                           float2* __restrict__ x1,
-                                                           const float2* __restrict__ twx,
-                                                           int W, int C, int m) {
-  extern __shared__ float sm[];
-  float2* tw = reinterpret_cast<float2*>(sm);  // W
-  float* tile = sm + 2 * W;                     // [32][C]
-  const size_t row = blockIdx.x;
-  for (int t = threadIdx.x; t < W; t += kSpecThreads) tw[t] = twx[t];
-  const int G = kSpecThreads / C;
-  const int c = threadIdx.x % C, g = threadIdx.x / C;
-  float2 acc[kAccMax];
-#pragma unroll
-  for (int k = 0; k < kAccMax; ++k) acc[k] = make_float2(0.f, 0.f);
-  for (int x0 = 0; x0 < W; x0 += 32) {
-    const int nx = min(32, W - x0);
     __syncthreads();
-    for (int j = threadIdx.x; j < nx * C; j += kSpecThreads)
-      tile[j] = f[(row * W + x0) * C + j];
-    __syncthreads();
-    if (g < G) {
+    float2 acc[PPT][4];
 #pragma unroll
-      for (int k = 0; k < kAccMax; ++k) {
-        const int kx = g + k * G;
-        if (kx < m) {
-          int idx = (kx * x0) % W;  // phase index (kx x) mod W, advanced by kx per x
-          for (int xx = 0; xx < nx; ++xx) {
-            const float2 e = tw[idx];
-            const float v = tile[xx * C + c];
-            acc[k].x = fmaf(v, e.x, acc[k].x);
-            acc[k].y = fmaf(-v, e.y, acc[k].y);
-            idx += kx;
-            if (idx >= W) idx -= W;
+    for (int i = 0; i < PPT; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+    auto sums = [&](const float* ar, const float* br, int bp, int n) {
+#pragma unroll 1
+      for (int k = 0; k < n; k += 4) {
+        float4 b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(br + j * G * bp + k);
+#pragma unroll
+        for (int i = 0; i < PPT; ++i) {
+          const float4 v = *reinterpret_cast<const float4*>(ar + i * NPG * ap + k);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            acc[i][j] = __ffma2_rn(make_float2(v.x, v.y), make_float2(b[j].x, b[j].y), acc[i][j]);
+            acc[i][j] = __ffma2_rn(make_float2(v.z, v.w), make_float2(b[j].z, b[j].w), acc[i][j]);
+          }
+        }
+      }
+    };
+    sums(A + pg * ap, Ws + og * wp, wp, cin4);
+    if (m2) sums(A + pg * ap + cin4, Zs + ((t / a.tpr) & 1) * OP * zp + og * zp, zp, m24);
+    __syncthreads();  // the buffers may be refilled
+    if (og * 4 < cout) {
+#pragma unroll
+      for (int i = 0; i < PPT; ++i) {
+        const int p = pg + i * NPG;
+        if (p >= np) continue;
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = (acc[i][j].x + acc[i][j].y) + bias[j];
+        const size_t at = (p0 + p) * cout + og * 4;
+        if (a.planar) {
+          const size_t b = (p0 + p) / a.hw, q = (p0 + p) - b * a.hw;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (og * 4 + j < cout) a.out[(b * cout + og * 4 + j) * a.hw + q] = v[j];
+        } else if ((cout & 3) == 0) {
+          if (a.pre) *reinterpret_cast<float4*>(a.pre + at) = make_float4(v[0], v[1], v[2], v[3]);
+          if (a.dz) {
+            const float4 d = *reinterpret_cast<const float4*>(a.dz + at);
+            v[0] *= tr_dact(d.x, a.act);
+            v[1] *= tr_dact(d.y, a.act);
+            v[2] *= tr_dact(d.z, a.act);
+            v[3] *= tr_dact(d.w, a.act);
+          } else if (a.out_act) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = tr_act(v[j], a.act);
+          }
+          *reinterpret_cast<float4*>(a.out + at) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (og * 4 + j >= cout) continue;
+            if (a.pre) a.pre[at + j] = v[j];
+            a.out[at + j] = a.dz ? v[j] * tr_dact(a.dz[at + j], a.act)
+                                 : (a.out_act ? tr_act(v[j], a.act) : v[j]);
           }
         }
       }
     }
   }
-  if (g < G) {
-#pragma unroll
-    for (int k = 0; k < kAccMax; ++k) {
-      const int kx = g + k * G;
-      if (kx < m) x1[(row * m + kx) * C + c] = acc[k];
+}
+
+// Block partials of dW[o][i] = sum_p dz[p][o] A(in[p][i]) and db[o] = sum_p dz[p][o] (pair
+// (o, cin) of the partial is db).  Block k covers a contiguous range of pixel tiles; a thread
+// owns 8 x 8 pairs (two quads along each axis) and one pixel in `groups`, the groups' sums are
+// added in order at the end.  FP32 multiply-adds bound it (32 packed ones for four shared loads);
+// stages are copied two ahead of use.
+struct WgArgs {
+  const float* dz;
+  const float* in;
+  float* part;
+  size_t P;
+  int cout, cin, in_act, act;
+};
+__device__ __forceinline__ void wg_load(const float* src, int n, int c, int pitch, float* dst) {
+  if ((c & 3) == 0) {
+    const int q = c >> 2;
+    for (int j = threadIdx.x; j < n * q; j += kWgThreads) {
+      const int p = j / q;
+      cpa16(dst + p * pitch + 4 * (j - p * q), src + 4 * j);
     }
+  } else {
+    for (int j = threadIdx.x; j < n * c; j += kWgThreads) {
+      const int p = j / c;
+      cpa4(dst + p * pitch + (j - p * c), src + j);
+    }
+  }
+}
+__global__ void __launch_bounds__(kWgThreads, 2) k_tr_wgrad(const WgArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  const int nto = (a.cout + 7) / 8, nti = (a.cin + 7) / 8;
+  const int dp = nto * 8, ip = nti * 8;             // row pitches
+  const int stage = kWgTile * (dp + ip);
+  const int tpg = nto * nti, groups = kWgThreads / tpg;
+  const int g = threadIdx.x / tpg, tg = threadIdx.x - g * tpg;
+  const int og = tg / nti, ig = tg - og * nti;
+  const int nbs = kWgThreads / dp, bo = threadIdx.x % dp, bs = threadIdx.x / dp;  // bias sums
+  const int npairs = a.cout * (a.cin + 1);
+  for (int j = threadIdx.x; j < 2 * stage; j += kWgThreads) sm[j] = 0.0f;  // pads stay 0
+  __syncthreads();
+  const size_t tiles = (a.P + kWgTile - 1) / kWgTile;
+  const size_t ta = tiles * blockIdx.x / gridDim.x, tb = tiles * (blockIdx.x + 1) / gridDim.x;
+  auto load = [&](size_t t, float* st) {
+    const size_t p0 = t * kWgTile;
+    const int n = (int)min((size_t)kWgTile, a.P - p0);
+    wg_load(a.dz + p0 * a.cout, n, a.cout, dp, st);
+    wg_load(a.in + p0 * a.cin, n, a.cin, ip, st + kWgTile * dp);
+  };
+  float2 acc[8][4];
+  float db = 0.0f;
+#pragma unroll
+  for (int o = 0; o < 8; ++o)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[o][i] = make_float2(0.0f, 0.0f);
+  if (ta < tb) load(ta, sm);
+  cpa_commit();
+  for (size_t t = ta; t < tb; ++t) {
+    float* st = sm + (t - ta & 1) * stage;
+    if (t + 1 < tb) load(t + 1, sm + ((t - ta + 1) & 1) * stage);
+    cpa_commit();
+    cpa_wait<1>();
+    __syncthreads();
+    const int n = (int)min((size_t)kWgTile, a.P - t * kWgTile);
+    float* is = st + kWgTile * dp;
+    if (a.in_act) {
+      for (int j = threadIdx.x; j < n * ip; j += kWgThreads) is[j] = tr_act(is[j], a.act);
+      __syncthreads();
+    }
+    if (g < groups) {
+#pragma unroll 2
+      for (int p = g; p < n; p += groups) {
+        const float* d = st + p * dp + og * 4;
+        const float* v = is + p * ip + ig * 4;
+        const float4 d0 = *reinterpret_cast<const float4*>(d);
+        const float4 d1 = *reinterpret_cast<const float4*>(d + nto * 4);
+        const float4 v0 = *reinterpret_cast<const float4*>(v);
+        const float4 v1 = *reinterpret_cast<const float4*>(v + nti * 4);
+        const float dd[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+        const float2 vv[4] = {make_float2(v0.x, v0.y), make_float2(v0.z, v0.w),
+                              make_float2(v1.x, v1.y), make_float2(v1.z, v1.w)};
+#pragma unroll
+        for (int o = 0; o < 8; ++o)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[o][i] = __ffma2_rn(dup2(dd[o]), vv[i], acc[o][i]);
+      }
+    }
+    if (bs < nbs)
+      for (int p = bs; p < n; p += nbs) db += st[p * dp + bo];
+    __syncthreads();
+  }
+  cpa_wait<0>();
+  __syncthreads();
+  // the groups' sums, in order
+  float* red = sm;  // [dp][ip + 1]
+  const int rp = ip + 1;
+  for (int j = threadIdx.x; j < dp * rp; j += kWgThreads) red[j] = 0.0f;
+  __syncthreads();
+  for (int q = 0; q < groups; ++q) {
+    if (g == q) {
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        const int oo = (o >> 2) * nto * 4 + og * 4 + (o & 3);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int ii = (i >> 1) * nti * 4 + ig * 4 + (i & 1) * 2;
+          red[oo * rp + ii] += acc[o][i].x;
+          red[oo * rp + ii + 1] += acc[o][i].y;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  for (int q = 0; q < nbs; ++q) {
+    if (bs == q) red[bo * rp + ip] += db;
+    __syncthreads();
+  }
+  float* out = a.part + (size_t)blockIdx.x * npairs;
+  for (int j = threadIdx.x; j < npairs; j += kWgThreads) {
+    const int o = j / (a.cin + 1), i = j - o * (a.cin + 1);
+    out[j] = red[o * rp + (i == a.cin ? ip : i)];
+  }
+}
+
+// Ordered sum of the block partials into dW (cout x cin) and db (cout): 32 pairs a block,
+// eight interleaved slices of the partials, in FP64.
+__global__ void __launch_bounds__(256) k_tr_wgrad_reduce(const float* __restrict__ part, int nblk,
+                                                         int cout, int cin, float* __restrict__ dw,
+                                                         float* __restrict__ db) {
+  __shared__ double red[8][32];
+  const int npairs = cout * (cin + 1);
+  const int l = threadIdx.x & 31, s = threadIdx.x >> 5;
+  const int pr = blockIdx.x * 32 + l;
+  double v = 0.0;
+  if (pr < npairs)
+    for (int k = s; k < nblk; k += 8) v += (double)part[(size_t)k * npairs + pr];
+  red[s][l] = v;
+  __syncthreads();
+  if (s == 0 && pr < npairs) {
+    for (int q = 1; q < 8; ++q) v += red[q][l];
+    const int o = pr / (cin + 1), i = pr - o * (cin + 1);
+    if (i == cin)
+      db[o] = (float)v;
+    else
+      dw[o * cin + i] = (float)v;
+  }
+}
+
+// Forward x-DFT: X1[row][kx][c] = sum_x f[row][x][c] e^{-2 pi i kx x / W}.  A block takes
+// kDftM (row, channel) pairs (whole rows' channels, padded to cp); a thread four channels x NP
+// frequencies (accumulators (Re, Im) packed) of every ks-th column; the column slices are
+// added in order.  Bound by FP32 multiply-adds and the one read of f; stages are double
+// buffered.
+template <int NP>
+__global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f,
+                                                     float2* __restrict__ x1,
+                                                     const float* __restrict__ ex, size_t rows,
+                                                     int W, int C, int cp, int m, int ng, int ks,
+                                                     int ep) {
+  extern __shared__ __align__(16) float sm[];
+  const int stage = kDftX * (kDftM + ep);
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int kg = wp % ng, sl = wp / ng;
+  const int rpb = kDftM / cp;
+  const size_t row0 = (size_t)blockIdx.x * rpb;
+  const int nr = (int)min((size_t)rpb, rows - row0);
+  const int nthr = blockDim.x;
+  auto load = [&](int x0, float* st) {
+    const int n = min(kDftX, W - x0);
+    for (int r = 0; r < nr; ++r) {
+      const float* src = f + ((row0 + r) * W + x0) * C;
+      if ((C & 3) == 0) {
+        const int q = C >> 2;
+        for (int j = threadIdx.x; j < n * q; j += nthr) {
+          const int x = j / q;
+          cpa16(st + x * kDftM + r * cp + 4 * (j - x * q), src + 4 * j);
+        }
+      } else {
+        for (int j = threadIdx.x; j < n * C; j += nthr) {
+          const int x = j / C;
+          cpa4(st + x * kDftM + r * cp + (j - x * C), src + j);
+        }
+      }
+    }
+    float* es = st + kDftX * kDftM;
+    for (int j = threadIdx.x; j < n * (ep >> 2); j += nthr) cpa16(es + 4 * j, ex + (size_t)x0 * ep + 4 * j);
+  };
+  float2 acc[4][NP];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int k = 0; k < NP; ++k) acc[j][k] = make_float2(0.0f, 0.0f);
+  load(0, sm);
+  cpa_commit();
+  int it = 0;
+  for (int x0 = 0; x0 < W; x0 += kDftX, it ^= 1) {
+    if (x0 + kDftX < W) load(x0 + kDftX, sm + (it ^ 1) * stage);
+    cpa_commit();
+    cpa_wait<1>();
+    __syncthreads();
+    const float* st = sm + it * stage;
+    const float* es = st + kDftX * kDftM + kg * 2 * NP;
+    const int n = min(kDftX, W - x0);
+#pragma unroll 2
+    for (int x = sl; x < n; x += ks) {
+      const float4 v = *reinterpret_cast<const float4*>(st + x * kDftM + 4 * lane);
+      const float2 d[4] = {dup2(v.x), dup2(v.y), dup2(v.z), dup2(v.w)};
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        const float2 e = *reinterpret_cast<const float2*>(es + x * ep + 2 * k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j][k] = __ffma2_rn(d[j], e, acc[j][k]);
+      }
+    }
+    __syncthreads();
+  }
+  cpa_wait<0>();
+  // the column slices, in order: slice q adds into (or starts) the block's sums
+  float2* red = reinterpret_cast<float2*>(sm);  // [NP ng][kDftM]
+  for (int q = 0; q < ks; ++q) {
+    if (sl == q) {
+#pragma unroll
+      for (int k = 0; k < NP; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float2* r = red + (kg * NP + k) * kDftM + 4 * lane + j;
+          if (q == 0)
+            *r = acc[j][k];
+          else
+            *r = make_float2(r->x + acc[j][k].x, r->y + acc[j][k].y);
+        }
+    }
+    __syncthreads();
+  }
+  for (int j = threadIdx.x; j < nr * m * C; j += nthr) {
+    const int r = j / (m * C), kx = j / C - r * m, c = j % C;
+    x1[((row0 + r) * m + kx) * C + c] = red[kx * kDftM + r * cp + c];
   }
 }
 
 // Forward y-DFT over the kept rows: Xh[b][a][kx][c] = scale(kx) sum_y X1[b][y][kx][c]
 // e^{-2 pi i ky(a) y / H}, ky(a) = a (a < m) or H - 2m + a; scale = 1, or c_kx / (H W)
-// for the adjoint of the real inverse transform.
-__global__ void __launch_bounds__(kSpecThreads) k_tr_dft_y(const float2* __restrict__ x1,
-                                                           float2* __restrict__ xh,
-                                                           const float2* __restrict__ twy,
-                                                           int H, int W, int C, int m,
-                                                           int adjoint_scale) {
-  extern __shared__ float sm[];
-  float2* tw = reinterpret_cast<float2*>(sm);  // H
-  float2* tile = tw + H;                        // [32][C]
-  const int b = blockIdx.x / m, kx = blockIdx.x % m;
-  for (int t = threadIdx.x; t < H; t += kSpecThreads) tw[t] = twy[t];
-  const int G = kSpecThreads / C;
-  const int c = threadIdx.x % C, g = threadIdx.x / C;
-  float2 acc[kAccMax];
+// for the adjoint of the real inverse transform.  A block takes one (b, kx) and kDftYA kept
+// rows; a lane two channels, a warp every eighth y; the warps' sums are added in order.
+__global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
+                                                  float2* __restrict__ xh,
+                                                  const float4* __restrict__ ey, int H, int W,
+                                                  int C, int m, int adjoint_scale) {
+  __shared__ float4 es[kDftYC][kDftYA];
+  __shared__ float4 red[kDftYA][32];
+  const int b = blockIdx.x / m, kx = blockIdx.x % m, a0 = blockIdx.y * kDftYA;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const bool on = 2 * lane < C;
+  float2 acc[kDftYA][2];
 #pragma unroll
-  for (int k = 0; k < kAccMax; ++k) acc[k] = make_float2(0.f, 0.f);
-  for (int y0 = 0; y0 < H; y0 += 32) {
-    const int ny = min(32, H - y0);
+  for (int a = 0; a < kDftYA; ++a) acc[a][0] = acc[a][1] = make_float2(0.0f, 0.0f);
+  for (int y0 = 0; y0 < H; y0 += kDftYC) {
     __syncthreads();
-    for (int j = threadIdx.x; j < ny * C; j += kSpecThreads) {
-      const int yy = j / C, cc = j - yy * C;
-      tile[j] = x1[(((size_t)b * H + y0 + yy) * m + kx) * C + cc];
+    for (int j = threadIdx.x; j < kDftYC * kDftYA; j += 256) {
+      const int y = y0 + j / kDftYA, a = a0 + j % kDftYA;
+      es[j / kDftYA][j % kDftYA] =
+          y < H && a < 2 * m ? ey[(size_t)y * 2 * m + a] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    if (g < G) {
+    const int n = min(kDftYC, H - y0);
+    if (on) {
+#pragma unroll 4
+      for (int y = wp; y < n; y += 8) {
+        const float4 v = *reinterpret_cast<const float4*>(
+            x1 + (((size_t)b * H + y0 + y) * m + kx) * C + 2 * lane);
 #pragma unroll
-      for (int k = 0; k < kAccMax; ++k) {
-        const int a = g + k * G;
-        if (a < 2 * m) {
-          const int ky = a < m ? a : H - 2 * m + a;
-          int idx = (int)(((long long)ky * y0) % H);  // (ky y) mod H, advanced by ky per y
-          for (int yy = 0; yy < ny; ++yy) {
-            const float2 e = tw[idx];  // e^{+i}: use conj
-            idx += ky;
-            if (idx >= H) idx -= H;
-            const float2 v = tile[yy * C + c];
-            // v * conj(e)
-            acc[k].x = fmaf(v.x, e.x, fmaf(v.y, e.y, acc[k].x));
-            acc[k].y = fmaf(v.y, e.x, fmaf(-v.x, e.y, acc[k].y));
-          }
+        for (int a = 0; a < kDftYA; ++a) {
+          const float4 e = es[y][a];
+          acc[a][0] = __ffma2_rn(dup2(v.x), make_float2(e.x, e.y), acc[a][0]);
+          acc[a][0] = __ffma2_rn(dup2(v.y), make_float2(e.z, e.w), acc[a][0]);
+          acc[a][1] = __ffma2_rn(dup2(v.z), make_float2(e.x, e.y), acc[a][1]);
+          acc[a][1] = __ffma2_rn(dup2(v.w), make_float2(e.z, e.w), acc[a][1]);
         }
       }
     }
   }
-  const float sc = adjoint_scale ? (kx == 0 ? 1.0f : 2.0f) / ((float)H * (float)W) : 1.0f;
-  if (g < G) {
+  for (int q = 0; q < 8; ++q) {
+    if (wp == q) {
 #pragma unroll
-    for (int k = 0; k < kAccMax; ++k) {
-      const int a = g + k * G;
-      if (a < 2 * m)
-        xh[(((size_t)b * 2 * m + a) * m + kx) * C + c] = make_float2(acc[k].x * sc, acc[k].y * sc);
+      for (int a = 0; a < kDftYA; ++a) {
+        float4 r = q ? red[a][lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        red[a][lane] = make_float4(r.x + acc[a][0].x, r.y + acc[a][0].y, r.z + acc[a][1].x,
+                                   r.w + acc[a][1].y);
+      }
     }
+    __syncthreads();
+  }
+  const float sc = adjoint_scale ? (kx == 0 ? 1.0f : 2.0f) / ((float)H * (float)W) : 1.0f;
+  const int a = wp;  // kDftYA == 8 warps
+  if (on && a0 + a < 2 * m) {
+    const float4 r = red[a][lane];
+    *reinterpret_cast<float4*>(xh + (((size_t)b * 2 * m + a0 + a) * m + kx) * C + 2 * lane) =
+        make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sc);
   }
 }
 
@@ -507,88 +816,57 @@ __global__ void k_tr_mix_bwd_r(const float2* __restrict__ xh, const float2* __re
   dparams[(lo ? r1im : r2im) + dst] = im;
 }
 
-// Inverse y-DFT: Z[b][y][kx][c] = sum_a Yh[b][a][kx][c] e^{+2 pi i ky(a) y / H}.
-__global__ void __launch_bounds__(kSpecThreads) k_tr_inv_y(const float2* __restrict__ yh,
-                                                           float2* __restrict__ z,
-                                                           const float2* __restrict__ twy,
-                                                           int H, int C, int m) {
-  extern __shared__ float sm[];
-  float2* tw = reinterpret_cast<float2*>(sm);  // H
-  float2* col = tw + H;                         // [2m][C]
-  const int b = blockIdx.x / m, kx = blockIdx.x % m;
-  for (int t = threadIdx.x; t < H; t += kSpecThreads) tw[t] = twy[t];
-  for (int j = threadIdx.x; j < 2 * m * C; j += kSpecThreads) {
-    const int a = j / C, c = j - a * C;
-    col[j] = yh[(((size_t)b * 2 * m + a) * m + kx) * C + c];
+// Inverse y-DFT: Z[b][y][kx][c] = w(kx) scale sum_a Yh[b][a][kx][c] e^{+2 pi i ky(a) y / H},
+// w(kx) = c_kx (forward) or 1 (adjoint of the forward DFT), ready for the pointwise kernel.  A
+// block takes one (b, kx) and 8 warps x kInvY rows; a lane two channels.
+__global__ void __launch_bounds__(256) k_tr_inv_y(const float2* __restrict__ yh,
+                                                  float2* __restrict__ z,
+                                                  const float4* __restrict__ ey, int H, int C,
+                                                  int m, float scale, int hermitian) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int YB = 8 * kInvY, EP = YB + 1;
+  float4* es = reinterpret_cast<float4*>(sm);       // [2m][EP]
+  float4* col = es + 2 * m * EP;                    // [2m][32]
+  const int b = blockIdx.x / m, kx = blockIdx.x % m, y0 = blockIdx.y * YB;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const bool on = 2 * lane < C;
+  for (int j = threadIdx.x; j < 2 * m * YB; j += 256) {
+    const int y = j / (2 * m), a = j - y * (2 * m);
+    es[a * EP + y] = y0 + y < H ? ey[(size_t)(y0 + y) * 2 * m + a] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  for (int j = threadIdx.x; j < 2 * m * 32; j += 256) {
+    const int a = j >> 5, l = j & 31;
+    if (2 * l < C)
+      col[j] = *reinterpret_cast<const float4*>(yh + (((size_t)b * 2 * m + a) * m + kx) * C + 2 * l);
   }
   __syncthreads();
-  const int G = kSpecThreads / C;
-  const int c = threadIdx.x % C, g = threadIdx.x / C;
-  if (g >= G) return;
-  for (int y = g; y < H; y += G) {
-    float re = 0.f, im = 0.f;
-    int idx = 0;  // (ky y) mod H for ky = 0 .. m-1, then H-m .. H-1
-    for (int a = 0; a < 2 * m; ++a) {
-      if (a == m) idx = (int)(((long long)(H - m) * y) % H);
-      const float2 e = tw[idx];
-      idx += y;
-      if (idx >= H) idx -= H;
-      const float2 v = col[a * C + c];
-      re = fmaf(v.x, e.x, fmaf(-v.y, e.y, re));
-      im = fmaf(v.x, e.y, fmaf(v.y, e.x, im));
+  if (!on) return;
+  float2 acc[kInvY][2];
+#pragma unroll
+  for (int y = 0; y < kInvY; ++y) acc[y][0] = acc[y][1] = make_float2(0.0f, 0.0f);
+#pragma unroll 2
+  for (int a = 0; a < 2 * m; ++a) {
+    const float4 v = col[a * 32 + lane];
+#pragma unroll
+    for (int y = 0; y < kInvY; ++y) {
+      const float4 e = es[a * EP + wp * kInvY + y];  // (c, -s, s, c); e^{+i phi}: (c, s, -s, c)
+      acc[y][0] = __ffma2_rn(dup2(v.x), make_float2(e.x, e.z), acc[y][0]);
+      acc[y][0] = __ffma2_rn(dup2(v.y), make_float2(e.y, e.w), acc[y][0]);
+      acc[y][1] = __ffma2_rn(dup2(v.z), make_float2(e.x, e.z), acc[y][1]);
+      acc[y][1] = __ffma2_rn(dup2(v.w), make_float2(e.y, e.w), acc[y][1]);
     }
-    z[(((size_t)b * H + y) * m + kx) * C + c] = make_float2(re, im);
+  }
+  const float w = (hermitian && kx > 0) ? 2.0f * scale : scale;
+#pragma unroll
+  for (int y = 0; y < kInvY; ++y) {
+    const int yy = y0 + wp * kInvY + y;
+    if (yy < H)
+      *reinterpret_cast<float4*>(z + (((size_t)b * H + yy) * m + kx) * C + 2 * lane) =
+          make_float4(acc[y][0].x * w, acc[y][0].y * w, acc[y][1].x * w, acc[y][1].y * w);
   }
 }
 
-// Inverse x-DFT with real output: S[row][x][c] = scale sum_kx w(kx) Re(Z[row][kx][c]
-// e^{+2 pi i kx x / W}); w(kx) = c_kx (forward) or 1 (adjoint of the forward DFT).
-__global__ void __launch_bounds__(kSpecThreads) k_tr_inv_x(const float2* __restrict__ z,
-                                                           float* __restrict__ s,
-                                                           const float2* __restrict__ twx,
-                                                           int W, int C, int m, float scale,
-                                                           int hermitian) {
-  extern __shared__ float sm[];
-  float2* tw = reinterpret_cast<float2*>(sm);  // W
-  float2* zr = tw + W;                          // [m][C]
-  const size_t row = blockIdx.x;
-  for (int t = threadIdx.x; t < W; t += kSpecThreads) tw[t] = twx[t];
-  for (int j = threadIdx.x; j < m * C; j += kSpecThreads) {
-    const int kx = j / C;
-    float2 v = z[row * m * C + j];
-    const float wk = (hermitian && kx > 0) ? 2.0f * scale : scale;
-    zr[j] = make_float2(v.x * wk, v.y * wk);
-  }
-  __syncthreads();
-  const int G = kSpecThreads / C;
-  const int c = threadIdx.x % C, g = threadIdx.x / C;
-  if (g >= G) return;
-  for (int x = g; x < W; x += G) {
-    float acc = 0.f;
-    int idx = 0;  // (kx x) mod W
-    for (int kx = 0; kx < m; ++kx) {
-      const float2 e = tw[idx];
-      idx += x;
-      if (idx >= W) idx -= W;
-      const float2 v = zr[kx * C + c];
-      acc = fmaf(v.x, e.x, fmaf(-v.y, e.y, acc));
-    }
-    s[(row * W + x) * C + c] = acc;
-  }
-}
-
-// NCHW <-> channels-last for the decoder output / its gradient
-__global__ void k_tr_cl_to_nchw(const float* __restrict__ cl, float* __restrict__ out, int B,
-                                int H, int W, int C) {
-  const size_t n = (size_t)B * C * H * W;
-  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const size_t hw = (size_t)H * W;
-  const int b = (int)(t / (C * hw));
-  const int c = (int)((t / hw) % C);
-  const size_t q = t % hw;
-  out[t] = cl[((size_t)b * hw + q) * C + c];
-}
+// planar -> channels-last for the gradient of the output
 __global__ void k_tr_nchw_to_cl(const float* __restrict__ in, float* __restrict__ cl, int B, int H,
                                 int W, int C) {
   const size_t n = (size_t)B * C * H * W;
@@ -624,74 +902,134 @@ struct TrCtx {
   unsigned char* ws;
 };
 
-size_t pw_smem(int cin, int cout) {
-  return sizeof(float) * ((size_t)cout * cin + (size_t)kPwPix * (cin + 1) + (size_t)kPwPix * (cout + 1));
+// A row pitch of at least n floats: an odd number of 16-byte units.
+int odd_pitch(int n) { return 4 * (((n + 3) / 4) | 1); }
+constexpr int pw_tile(int op) { return op == 64 ? 64 : 128; }
+struct PwSmem {
+  int ap, wp, zp;
+  size_t bytes;
+};
+PwSmem pw_smem(int op, int cin, int m) {
+  PwSmem r;
+  r.ap = odd_pitch((cin + 3) / 4 * 4 + 2 * m);
+  r.wp = odd_pitch(cin);
+  r.zp = m ? odd_pitch(2 * m) : 0;
+  r.bytes = sizeof(float) * ((size_t)2 * pw_tile(op) * r.ap + (size_t)op * (r.wp + 2 * r.zp));
+  return r;
 }
-
-int pw(const TrCtx& x, const float* in, int cin, const float* w, int trans, const float* bias,
-       const float* add, int cout, float* pre, float* out, int in_act, int out_act) {
-  const size_t smem = pw_smem(cin, cout);
-  k_tr_pw<<<nb(x.pl.P, kPwPix), kPwPix, smem, x.st>>>(in, cin, w, trans, bias, add, cout, pre, out,
-                                                      in_act, out_act, x.c->activation, x.pl.P);
+template <int OP>
+int pw_run(const TrCtx& x, PwArgs a) {
+  constexpr int PT = pw_tile(OP);
+  const PwSmem sm = pw_smem(OP, a.cin, a.z ? a.m : 0);
+  a.ap = sm.ap;
+  a.wp = sm.wp;
+  a.zp = sm.zp;
+  a.tpr = (a.W + PT - 1) / PT;
+  a.ntiles = a.z ? x.B * x.H * a.tpr : (int)((a.P + PT - 1) / PT);
+  const int ctas = std::max(1, std::min<int>(kPwCtas, (int)((227 << 10) / (sm.bytes + 1024))));
+  k_tr_pw<OP, PT><<<std::min(a.ntiles, ctas * kTrSms), kPwThreads, sm.bytes, x.st>>>(a);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
+// What one pointwise launch does besides its layer (PwArgs).
+struct PwOpt {
+  const float2* z = nullptr;
+  const float* dz = nullptr;
+  float* pre = nullptr;
+  int in_act = 0, out_act = 0, planar = 0;
+};
+int pw(const TrCtx& x, const float* in, int cin, const float* w, int trans, const float* bias,
+       int cout, float* out, const PwOpt& o = PwOpt{}) {
+  PwArgs a{};
+  a.in = in;
+  a.w = w;
+  a.bias = bias;
+  a.z = o.z;
+  a.ex = reinterpret_cast<const float*>(x.ws + x.pl.ex);
+  a.dz = o.dz;
+  a.pre = o.pre;
+  a.out = out;
+  a.P = x.pl.P;
+  a.hw = (size_t)x.H * x.W;
+  a.cin = cin;
+  a.cout = cout;
+  a.trans = trans;
+  a.in_act = o.in_act;
+  a.out_act = o.out_act;
+  a.act = x.c->activation;
+  a.planar = o.planar;
+  a.W = x.W;
+  a.m = x.c->modes;
+  a.ep = x.pl.ep;
+  // output columns of a block: the smallest tile that holds them
+  return cout > 32 ? pw_run<64>(x, a) : (cout > 16 ? pw_run<32>(x, a) : pw_run<16>(x, a));
+}
 
+size_t wg_smem(int cout, int cin) {
+  const size_t dp = (cout + 7) / 8 * 8, ip = (cin + 7) / 8 * 8;
+  return sizeof(float) * std::max(2 * kWgTile * (dp + ip), dp * (ip + 1));
+}
 int wgrad(const TrCtx& x, const float* dz, int cout, const float* in, int cin, int in_act,
           float* dw, float* db) {
   float* part = reinterpret_cast<float*>(x.ws + x.pl.part);
-  k_tr_wgrad<<<x.pl.wg_blocks, kWgThreads, 0, x.st>>>(dz, cout, in, cin, in_act,
-                                                      x.c->activation, x.pl.P, part);
+  const WgArgs a{dz, in, part, x.pl.P, cout, cin, in_act, x.c->activation};
+  k_tr_wgrad<<<x.pl.wg_blocks, kWgThreads, wg_smem(cout, cin), x.st>>>(a);
   LBM_CHECK_LAUNCH();
-  k_tr_wgrad_reduce<<<nb((size_t)cout * (cin + 1)), 256, 0, x.st>>>(part, x.pl.wg_blocks, cout,
-                                                                    cin, dw, db);
+  k_tr_wgrad_reduce<<<nb((size_t)cout * (cin + 1), 32), 256, 0, x.st>>>(part, x.pl.wg_blocks, cout,
+                                                                        cin, dw, db);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
 
 // X (or the adjoint-scaled dY) of a field: forward x-DFT then y-DFT over the kept rows.
+size_t dft_x_smem(int ep, int np, int ng) {
+  return std::max(sizeof(float) * 2 * kDftX * (kDftM + ep), sizeof(float2) * kDftM * np * ng);
+}
 int spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_scale) {
-  const int C = x.c->width, m = x.c->modes;
+  const int C = x.c->width, m = x.c->modes, np = x.pl.np, ng = x.pl.ng, ep = x.pl.ep;
   float2* x1 = reinterpret_cast<float2*>(x.ws + x.pl.x1);
-  const float2* twx = reinterpret_cast<const float2*>(x.ws + x.pl.twx);
-  const float2* twy = reinterpret_cast<const float2*>(x.ws + x.pl.twy);
-  k_tr_dft_x<<<x.B * x.H, kSpecThreads, (2 * x.W + 32 * C) * sizeof(float), x.st>>>(f, x1, twx, x.W,
-                                                                                    C, m);
+  const int cp = C <= 8 ? 8 : (C <= 16 ? 16 : (C <= 32 ? 32 : 64));
+  const int ks = std::max(1, 8 / ng);
+  const size_t rows = (size_t)x.B * x.H;
+  auto kernel = np == 4 ? k_tr_dft_x<4> : (np == 6 ? k_tr_dft_x<6> : (np == 7 ? k_tr_dft_x<7>
+                                                                              : k_tr_dft_x<8>));
+  kernel<<<nb(rows, kDftM / cp), 32 * ng * ks, dft_x_smem(ep, np, ng), x.st>>>(
+      f, x1, reinterpret_cast<const float*>(x.ws + x.pl.ex), rows, x.W, C, cp, m, ng, ks, ep);
   LBM_CHECK_LAUNCH();
-  k_tr_dft_y<<<x.B * m, kSpecThreads, (x.H + 32 * C) * sizeof(float2), x.st>>>(
-      x1, out, twy, x.H, x.W, C, m, adjoint_scale);
+  k_tr_dft_y<<<dim3(x.B * m, nb(2 * m, kDftYA)), 256, 0, x.st>>>(
+      x1, out, reinterpret_cast<const float4*>(x.ws + x.pl.ey), x.H, x.W, C, m, adjoint_scale);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
 
-// Real field from kept coefficients: inverse y-DFT then inverse x-DFT.
-int spectral_inv(const TrCtx& x, const float2* coef, float* s, float scale, int hermitian) {
+// Row coefficients from kept coefficients: the inverse y-DFT (the pointwise kernel does the
+// rest of the inverse).
+size_t inv_y_smem(int m) { return sizeof(float4) * 2 * m * (8 * kInvY + 1 + 32); }
+int spectral_inv(const TrCtx& x, const float2* coef, float scale, int hermitian) {
   const int C = x.c->width, m = x.c->modes;
-  float2* z = reinterpret_cast<float2*>(x.ws + x.pl.z);
-  const float2* twx = reinterpret_cast<const float2*>(x.ws + x.pl.twx);
-  const float2* twy = reinterpret_cast<const float2*>(x.ws + x.pl.twy);
-  k_tr_inv_y<<<x.B * m, kSpecThreads, (x.H + 2 * m * C) * sizeof(float2), x.st>>>(coef, z, twy,
-                                                                                  x.H, C, m);
-  LBM_CHECK_LAUNCH();
-  k_tr_inv_x<<<x.B * x.H, kSpecThreads, (x.W + m * C) * sizeof(float2), x.st>>>(z, s, twx, x.W, C, m,
-                                                                                scale, hermitian);
+  k_tr_inv_y<<<dim3(x.B * m, nb(x.H, 8 * kInvY)), 256, inv_y_smem(m), x.st>>>(
+      coef, reinterpret_cast<float2*>(x.ws + x.pl.z),
+      reinterpret_cast<const float4*>(x.ws + x.pl.ey), x.H, C, m, scale, hermitian);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
 
+template <typename K>
+cudaError_t smem_limit(K k, size_t bytes) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 int set_smem_limits() {
   static bool done = false;
   if (done) return LBM_OK;
-  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_tr_pw, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)pw_smem(64, 64)));
-  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_tr_dft_x, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((2 * 2048 + 32 * 64) * sizeof(float))));
-  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_tr_dft_y, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((8192 + 32 * 64) * sizeof(float2))));
-  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_tr_inv_y, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((8192 + 2 * kTrModesMax * 64) * sizeof(float2))));
-  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_tr_inv_x, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((2048 + kTrModesMax * 64) * sizeof(float2))));
+  LBM_CHECK_CUDA(smem_limit(k_tr_pw<64, pw_tile(64)>, pw_smem(64, 64, kTrModesMax).bytes));
+  LBM_CHECK_CUDA(smem_limit(k_tr_pw<32, pw_tile(32)>, pw_smem(32, 64, kTrModesMax).bytes));
+  LBM_CHECK_CUDA(smem_limit(k_tr_pw<16, pw_tile(16)>, pw_smem(16, 64, kTrModesMax).bytes));
+  LBM_CHECK_CUDA(smem_limit(k_tr_wgrad, wg_smem(64, 64)));
+  LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<4>, dft_x_smem(64, 8, 4)));
+  LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<6>, dft_x_smem(72, 8, 5)));
+  LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<7>, dft_x_smem(72, 8, 5)));
+  LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<8>, dft_x_smem(64, 8, 4)));
+  LBM_CHECK_CUDA(smem_limit(k_tr_inv_y, inv_y_smem(kTrModesMax)));
   done = true;
   return LBM_OK;
 }
@@ -712,9 +1050,11 @@ int tr_setup(const fno_config* cfg, const float* params, int B, int H, int W, vo
   x->W = W;
   x->st = TS(stream);
   x->ws = static_cast<unsigned char*>(ws);
-  k_tr_twiddle<<<nb(W), 256, 0, x->st>>>(reinterpret_cast<float2*>(x->ws + x->pl.twx), W);
+  k_tr_ex<<<nb((size_t)W * x->pl.ep / 2), 256, 0, x->st>>>(
+      reinterpret_cast<float*>(x->ws + x->pl.ex), W, cfg->modes, x->pl.ep);
   LBM_CHECK_LAUNCH();
-  k_tr_twiddle<<<nb(H), 256, 0, x->st>>>(reinterpret_cast<float2*>(x->ws + x->pl.twy), H);
+  k_tr_ey<<<nb((size_t)H * 2 * cfg->modes), 256, 0, x->st>>>(
+      reinterpret_cast<float4*>(x->ws + x->pl.ey), H, cfg->modes);
   LBM_CHECK_LAUNCH();
   // spectral filters per layer, transposed to [mode][i][o]
   RtOffs offs{};
@@ -770,37 +1110,35 @@ int fno_train_forward(const fno_config* cfg_h, const float* params_d, const floa
   auto zpre = [&](int n) { return saved_d + pl.zpre + (size_t)n * P * C; };
   auto xh = [&](int n) { return reinterpret_cast<float2*>(saved_d + pl.xh) + (size_t)n * spec; };
   auto hdpre = [&](int l) { return saved_d + pl.hdpre + (size_t)l * P * S; };
-  float* ta = reinterpret_cast<float*>(x.ws + pl.ta);
-  float* tb = reinterpret_cast<float*>(x.ws + pl.tb);
-  float* s = reinterpret_cast<float*>(x.ws + pl.s);
   float2* yh = reinterpret_cast<float2*>(x.ws + pl.yh);
+  const float2* z = reinterpret_cast<const float2*>(x.ws + pl.z);
   const float2* rt = reinterpret_cast<const float2*>(x.ws + pl.rt);
   const float* p = params_d;
 
   k_tr_xin<<<nb(P), 256, 0, x.st>>>(in_d, xin, B, H, W, c.c_in);
   LBM_CHECK_LAUNCH();
-  LBM_TRY(pw(x, xin, c.c_in + 2, p + o.lift0_w, 0, p + o.lift0_b, nullptr, h, h1pre, ta, 0, 1));
-  LBM_TRY(pw(x, ta, h, p + o.lift1_w, 0, p + o.lift1_b, nullptr, C, nullptr, theta(0), 0, 0));
+  // hidden layers store their pre-activations only; the next layer applies sigma as it reads
+  LBM_TRY(pw(x, xin, c.c_in + 2, p + o.lift0_w, 0, p + o.lift0_b, h, h1pre));
+  PwOpt act_in;
+  act_in.in_act = 1;
+  LBM_TRY(pw(x, h1pre, h, p + o.lift1_w, 0, p + o.lift1_b, C, theta(0), act_in));
   for (int n = 0; n < c.layers; ++n) {
     LBM_TRY(spectral_fwd(x, theta(n), xh(n), 0));
     k_tr_mix<<<nb(spec), 256, 0, x.st>>>(xh(n), rt + (size_t)n * 2 * m * m * C * C, yh, B, C,
                                          2 * m * m);
     LBM_CHECK_LAUNCH();
-    LBM_TRY(spectral_inv(x, yh, s, 1.0f / ((float)H * (float)W), 1));
-    LBM_TRY(pw(x, theta(n), C, p + o.w[n], 0, p + o.b[n], s, C, zpre(n), theta(n + 1), 0, 1));
+    LBM_TRY(spectral_inv(x, yh, 1.0f / ((float)H * (float)W), 1));
+    PwOpt opt;
+    opt.z = z;
+    opt.pre = zpre(n);
+    opt.out_act = 1;
+    LBM_TRY(pw(x, theta(n), C, p + o.w[n], 0, p + o.b[n], C, theta(n + 1), opt));
   }
-  const float* hin = theta(c.layers);
-  int fan = C;
-  for (int l = 0; l < c.dec_layers; ++l) {
-    float* hout = (l % 2 == 0) ? ta : tb;
-    LBM_TRY(pw(x, hin, fan, p + o.dec_w[l], 0, p + o.dec_b[l], nullptr, S, hdpre(l), hout, 0, 1));
-    hin = hout;
-    fan = S;
-  }
-  float* ycl = reinterpret_cast<float*>(x.ws + pl.ycl);
-  LBM_TRY(pw(x, hin, fan, p + o.out_w, 0, p + o.out_b, nullptr, c.c_out, nullptr, ycl, 0, 0));
-  k_tr_cl_to_nchw<<<nb(P * c.c_out), 256, 0, x.st>>>(ycl, out_d, B, H, W, c.c_out);
-  LBM_CHECK_LAUNCH();
+  for (int l = 0; l < c.dec_layers; ++l)
+    LBM_TRY(pw(x, l == 0 ? theta(c.layers) : hdpre(l - 1), l == 0 ? C : S, p + o.dec_w[l], 0,
+               p + o.dec_b[l], S, hdpre(l), l == 0 ? PwOpt{} : act_in));
+  act_in.planar = 1;
+  LBM_TRY(pw(x, hdpre(c.dec_layers - 1), S, p + o.out_w, 0, p + o.out_b, c.c_out, out_d, act_in));
   return LBM_OK;
 }
 
@@ -814,7 +1152,7 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
   const fno_config& c = *cfg_h;
   const TrPlan& pl = x.pl;
   const TrOff& o = x.off;
-  const int C = c.width, h = C / 2, S = c.dec_size, m = c.modes, act = c.activation;
+  const int C = c.width, h = C / 2, S = c.dec_size, m = c.modes;
   const size_t P = pl.P, spec = (size_t)B * 2 * m * m * C;
   const float* xin = saved_d + pl.xin;
   const float* h1pre = saved_d + pl.h1pre;
@@ -826,8 +1164,6 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
   auto hdpre = [&](int l) { return saved_d + pl.hdpre + (size_t)l * P * S; };
   float* ta = reinterpret_cast<float*>(x.ws + pl.ta);
   float* tb = reinterpret_cast<float*>(x.ws + pl.tb);
-  float* dz = reinterpret_cast<float*>(x.ws + pl.dz);
-  float* s = reinterpret_cast<float*>(x.ws + pl.s);
   float2* dyh = reinterpret_cast<float2*>(x.ws + pl.dyh);
   float2* dxh = reinterpret_cast<float2*>(x.ws + pl.yh);
   const float2* rt = reinterpret_cast<const float2*>(x.ws + pl.rt);
@@ -839,47 +1175,48 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
   k_tr_nchw_to_cl<<<nb(P * c.c_out), 256, 0, x.st>>>(dout_d, ycl, B, H, W, c.c_out);
   LBM_CHECK_LAUNCH();
   const int L = c.dec_layers;
-  const int fan_last = S;
-  LBM_TRY(wgrad(x, ycl, c.c_out, hdpre(L - 1), fan_last, 1, dp + o.out_w, dp + o.out_b));
-  LBM_TRY(pw(x, ycl, c.c_out, p + o.out_w, 1, nullptr, nullptr, fan_last, nullptr, ta, 0, 0));
-  float* g = ta;  // gradient with respect to the output of decoder layer L-1
+  // g: gradient with respect to the pre-activation of the layer at hand, in ta or tb
+  LBM_TRY(wgrad(x, ycl, c.c_out, hdpre(L - 1), S, 1, dp + o.out_w, dp + o.out_b));
+  PwOpt opt;
+  opt.dz = hdpre(L - 1);
+  LBM_TRY(pw(x, ycl, c.c_out, p + o.out_w, 1, nullptr, S, ta, opt));
+  float* g = ta;
   for (int l = L - 1; l >= 0; --l) {
-    k_tr_act_bwd<<<nb(P * S), 256, 0, x.st>>>(g, hdpre(l), dz, P * S, act);
-    LBM_CHECK_LAUNCH();
     const float* lin = (l == 0) ? theta(c.layers) : hdpre(l - 1);
     const int fan = (l == 0) ? C : S;
-    LBM_TRY(wgrad(x, dz, S, lin, fan, l == 0 ? 0 : 1, dp + o.dec_w[l], dp + o.dec_b[l]));
+    LBM_TRY(wgrad(x, g, S, lin, fan, l == 0 ? 0 : 1, dp + o.dec_w[l], dp + o.dec_b[l]));
     float* gn = (g == ta) ? tb : ta;
-    LBM_TRY(pw(x, dz, S, p + o.dec_w[l], 1, nullptr, nullptr, fan, nullptr, gn, 0, 0));
+    opt.dz = (l == 0) ? zpre(c.layers - 1) : hdpre(l - 1);
+    LBM_TRY(pw(x, g, S, p + o.dec_w[l], 1, nullptr, fan, gn, opt));
     g = gn;
   }
-  // Fourier layers in reverse: g = dL/dtheta_{n+1}
+  // Fourier layers in reverse: g = dz_n
   for (int n = c.layers - 1; n >= 0; --n) {
-    k_tr_act_bwd<<<nb(P * C), 256, 0, x.st>>>(g, zpre(n), dz, P * C, act);
-    LBM_CHECK_LAUNCH();
-    LBM_TRY(wgrad(x, dz, C, theta(n), C, 0, dp + o.w[n], dp + o.b[n]));
-    LBM_TRY(spectral_fwd(x, dz, dyh, 1));
+    LBM_TRY(wgrad(x, g, C, theta(n), C, 0, dp + o.w[n], dp + o.b[n]));
+    LBM_TRY(spectral_fwd(x, g, dyh, 1));
     k_tr_mix_bwd_r<<<nb((size_t)2 * m * m * C * C), 256, 0, x.st>>>(
         xh(n), dyh, dp, o.r1re[n], o.r1im[n], o.r2re[n], o.r2im[n], B, C, m);
     LBM_CHECK_LAUNCH();
     k_tr_mix_bwd_x<<<nb(spec), 256, 0, x.st>>>(dyh, rt + (size_t)n * 2 * m * m * C * C, dxh, B, C,
                                                2 * m * m);
     LBM_CHECK_LAUNCH();
-    LBM_TRY(spectral_inv(x, dxh, s, 1.0f, 0));
+    LBM_TRY(spectral_inv(x, dxh, 1.0f, 0));
     float* gn = (g == ta) ? tb : ta;
-    LBM_TRY(pw(x, dz, C, p + o.w[n], 1, nullptr, s, C, nullptr, gn, 0, 0));
+    PwOpt lo;
+    lo.z = reinterpret_cast<const float2*>(x.ws + pl.z);
+    lo.dz = n > 0 ? zpre(n - 1) : nullptr;
+    LBM_TRY(pw(x, g, C, p + o.w[n], 1, nullptr, C, gn, lo));
     g = gn;
   }
   // lifting network: g = dL/dtheta_0
   LBM_TRY(wgrad(x, g, C, h1pre, h, 1, dp + o.lift1_w, dp + o.lift1_b));
   float* gh = (g == ta) ? tb : ta;
-  LBM_TRY(pw(x, g, C, p + o.lift1_w, 1, nullptr, nullptr, h, nullptr, gh, 0, 0));
-  k_tr_act_bwd<<<nb(P * h), 256, 0, x.st>>>(gh, h1pre, dz, P * h, act);
-  LBM_CHECK_LAUNCH();
-  LBM_TRY(wgrad(x, dz, h, xin, c.c_in + 2, 0, dp + o.lift0_w, dp + o.lift0_b));
+  opt.dz = h1pre;
+  LBM_TRY(pw(x, g, C, p + o.lift1_w, 1, nullptr, h, gh, opt));
+  LBM_TRY(wgrad(x, gh, h, xin, c.c_in + 2, 0, dp + o.lift0_w, dp + o.lift0_b));
   if (din_d) {
     float* gx = (gh == ta) ? tb : ta;
-    LBM_TRY(pw(x, dz, h, p + o.lift0_w, 1, nullptr, nullptr, c.c_in + 2, nullptr, gx, 0, 0));
+    LBM_TRY(pw(x, gh, h, p + o.lift0_w, 1, nullptr, c.c_in + 2, gx));
     k_tr_din<<<nb(P * c.c_in), 256, 0, x.st>>>(gx, din_d, B, H, W, c.c_in);
     LBM_CHECK_LAUNCH();
   }
