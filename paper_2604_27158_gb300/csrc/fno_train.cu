@@ -2,8 +2,8 @@
 // reverse mode) for GB300 (sm_103a) and their C ABI.
 //
 // The training path keeps FP32 master parameters and FP32 activations: the forward
-// pass saves, per layer, the latent field theta_n, the pre-activation z_n and the
-// kept spectral coefficients X_n = F(theta_n); the backward pass is the chain rule
+// pass saves, per layer, the latent field theta_n, the derivative sigma'(z_n) of its
+// activation (zpre below) and the kept spectral coefficients X_n = F(theta_n); the backward pass is the chain rule
 // through the same operators, with the spectral layer's adjoint written out:
 //   z = W theta + b + F^-1(R . F(theta)),   theta' = sigma(z)
 //   dz      = dtheta' * sigma'(z)
@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "gelu_train_poly.cuh"
 
 namespace lbmfno {
 
@@ -33,8 +34,7 @@ inline cudaStream_t TS(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 constexpr int kTrModesMax = 32;
 constexpr int kTrSms = 152;
-constexpr int kPwThreads = 256;  // threads of the pointwise kernel
-constexpr int kPwCtas = 3;       // its blocks a multiprocessor (shared memory, registers)
+__host__ __device__ constexpr int pw_ctas(int threads) { return 512 / threads; }  // 128 registers
 constexpr int kWgThreads = 256;  // threads of the weight-gradient kernel
 constexpr int kWgTile = 64;      // pixels of one of its stages
 constexpr int kDftM = 128;       // (row, channel) pairs of an x-DFT block
@@ -157,17 +157,54 @@ TrPlan tr_plan(const fno_config& c, int B, int H, int W) {
   return t;
 }
 
-__device__ __forceinline__ float tr_act(float v, int act) {
-  return act == FNO_ACT_GELU ? 0.5f * v * (1.0f + erff(v * 0.70710678118654752f))
-                             : fmaxf(v, 0.0f);
+// sigma(v) and sigma'(v) of two values: GELU v Phi(v) and Phi(v) + v phi(v), or ReLU and the
+// step function.  With a = |v|, e = exp(-a^2 / 2) and Q = Phi(-a) = e S(a) (gelu_train_poly.cuh):
+//   v Phi(v) = max(v, 0) - a Q,   sigma'(v) = 1 - r for v >= 0, r else, r = e (S - a / sqrt(2 pi)).
+// Packed FP32, one ex2.approx a value; as accurate as the erf form in FP32 (2.4e-7 at most, 1.8e-8
+// rms on normal values, against 4.5e-7 and 2.4e-8; the derivative 2.6e-8 rms, against 2.6e-8).  The
+// erf form took as many issue slots as the 64-channel layer it follows.  NaN propagates.
+__device__ __forceinline__ void tr_gelu2(float2 v, float2* g, float2* d) {
+  constexpr float c[GELU_T_DEG + 1] = GELU_T_COEFFS;
+  // beyond 64 the tail is 0; the clamp keeps a Q defined for infinities
+  const float2 a = make_float2(fminf(fabsf(v.x), 64.0f), fminf(fabsf(v.y), 64.0f));
+  const float2 u = __ffma2_rn(make_float2(fminf(a.x, 6.0f), fminf(a.y, 6.0f)),
+                              make_float2(1.0f / 3.0f, 1.0f / 3.0f), make_float2(-1.0f, -1.0f));
+  float2 p = make_float2(c[GELU_T_DEG], c[GELU_T_DEG]);
+#pragma unroll
+  for (int k = GELU_T_DEG - 1; k >= 0; --k) p = __ffma2_rn(p, u, make_float2(c[k], c[k]));
+  const float2 t = __fmul2_rn(__fmul2_rn(a, a), make_float2(-0.72134752044448170f, -0.72134752044448170f));
+  float2 e;  // 2^t = exp(-a^2 / 2)
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(t.x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(t.y));
+  float2 h;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(h.x) : "f"(v.x));
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(h.y) : "f"(v.y));
+  const float2 na = make_float2(-a.x, -a.y);
+  if (g) *g = __ffma2_rn(na, __fmul2_rn(e, p), h);
+  if (d) {
+    const float2 r = __fmul2_rn(e, __ffma2_rn(na, make_float2(0.39894228040143268f, 0.39894228040143268f), p));
+    // a NaN compares false with both: v itself
+    *d = make_float2(v.x >= 0.0f ? 1.0f - r.x : (v.x < 0.0f ? r.x : v.x),
+                     v.y >= 0.0f ? 1.0f - r.y : (v.y < 0.0f ? r.y : v.y));
+  }
 }
-// sigma'(v): GELU Phi(v) + v phi(v); ReLU the step function
-__device__ __forceinline__ float tr_dact(float v, int act) {
-  if (act != FNO_ACT_GELU) return v > 0.0f ? 1.0f : 0.0f;
-  const float cdf = 0.5f * (1.0f + erff(v * 0.70710678118654752f));
-  const float pdf = 0.39894228040143268f * expf(-0.5f * v * v);
-  return cdf + v * pdf;
+__device__ __forceinline__ float2 tr_act2(float2 v, int act) {
+  if (act != FNO_ACT_GELU) return make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f));
+  float2 g;
+  tr_gelu2(v, &g, nullptr);
+  return g;
 }
+__device__ __forceinline__ float2 tr_dact2(float2 v, int act) {
+  if (act != FNO_ACT_GELU) return make_float2(v.x > 0.0f ? 1.0f : 0.0f, v.y > 0.0f ? 1.0f : 0.0f);
+  float2 d;
+  tr_gelu2(v, nullptr, &d);
+  return d;
+}
+__device__ __forceinline__ float4 tr_act4(float4 v, int act) {
+  const float2 a = tr_act2(make_float2(v.x, v.y), act), b = tr_act2(make_float2(v.z, v.w), act);
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ float tr_act(float v, int act) { return tr_act2(make_float2(v, v), act).x; }
 __device__ __forceinline__ float bf16r(float v) {
   return __bfloat162float(__float2bfloat16_rn(v));
 }
@@ -259,12 +296,31 @@ template <int N>
 __device__ __forceinline__ void cpa_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+// Walks j = threadIdx.x, + n, ... over rows of `len` items as (row r, item c) with one division.
+struct Walk {
+  int r, c, dr, dc, len;
+  __device__ __forceinline__ Walk(int n, int len_) : len(len_) {
+    r = (int)threadIdx.x / len;
+    c = (int)threadIdx.x - r * len;
+    dr = n / len;
+    dc = n - dr * len;
+  }
+  __device__ __forceinline__ void next() {
+    r += dr;
+    c += dc;
+    if (c >= len) {
+      c -= len;
+      ++r;
+    }
+  }
+};
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 
 // Pointwise linear layer, with the inverse x-DFT of a row's coefficients added:
 //   v[p][o] = bias[o] + sum_i Wm(o, i) A(in[p][i]) + sum_kx Re(z[row][kx][o] e^{+2 pi i kx x / W}),
 //   Wm(o, i) = trans ? w[i * cout + o] : w[o * cin + i],  A = sigma if in_act else identity;
-//   pre[p][o] = v (if pre);  out[p][o] = sigma(v) if out_act, v * sigma'(dz[p][o]) if dz, else v
+//   pre[p][o] = sigma'(v) (if pre);  out[p][o] = sigma(v) if out_act, v * d[p][o] if d,
+//   v * sigma'(dz[p][o]) if dz, else v
 // (planar: out is [b][cout][hw]).  One contraction over cin + 2m terms: the columns of A are
 // the inputs and the (cos, -sin) table of the pixel's column, those of B the weights and the
 // row's coefficients (Re, Im).
@@ -281,6 +337,7 @@ struct PwArgs {
   const float* bias;
   const float2* z;   // [row][m][cout], or null
   const float* ex;
+  const float* d;
   const float* dz;
   float* pre;
   float* out;
@@ -290,9 +347,9 @@ struct PwArgs {
   int ap, wp, zp;    // row pitches: inputs, weights, coefficients
   int ntiles, tpr;   // tiles; tiles a row (z)
 };
-template <int OP, int PT>
-__global__ void __launch_bounds__(kPwThreads, kPwCtas) k_tr_pw(const PwArgs a) {
-  constexpr int G = OP / 4, NPG = kPwThreads / G, PPT = PT / NPG;
+template <int OP, int PT, int NT>
+__global__ void __launch_bounds__(NT, pw_ctas(NT)) k_tr_pw(const PwArgs a) {
+  constexpr int G = OP / 4, NPG = NT / G, PPT = PT / NPG;
   static_assert(PPT >= 1 && NPG * PPT == PT, "pixels a thread");
   extern __shared__ __align__(16) float sm[];
   float* As = sm;                       // [2][PT][ap]: inputs, then the table's columns
@@ -300,9 +357,9 @@ __global__ void __launch_bounds__(kPwThreads, kPwCtas) k_tr_pw(const PwArgs a) {
   float* Zs = Ws + OP * a.wp;           // [2][OP][zp], rows as Ws
   const int ap = a.ap, wp = a.wp, zp = a.zp, cin = a.cin, cout = a.cout;
   const int cin4 = (cin + 3) & ~3, m2 = a.z ? 2 * a.m : 0, m24 = (m2 + 3) & ~3;
-  for (int j = threadIdx.x; j < 2 * PT * ap + OP * (wp + 2 * zp); j += kPwThreads) sm[j] = 0.0f;
+  for (int j = threadIdx.x; j < 2 * PT * ap + OP * (wp + 2 * zp); j += NT) sm[j] = 0.0f;
   __syncthreads();
-  for (int j = threadIdx.x; j < cout * cin; j += kPwThreads) {
+  for (int j = threadIdx.x; j < cout * cin; j += NT) {
     const int o = a.trans ? j % cout : j / cin, i = a.trans ? j / cout : j - o * cin;
     Ws[((o & 3) * G + (o >> 2)) * wp + i] = a.w[j];
   }
@@ -325,37 +382,30 @@ __global__ void __launch_bounds__(kPwThreads, kPwCtas) k_tr_pw(const PwArgs a) {
       np = (int)min((size_t)PT, a.P - p0);
     }
   };
+  // items of a pixel's inputs as they are copied: four channels, or one
+  const bool quad = (cin & 3) == 0;
+  const Walk wa(NT, quad ? cin >> 2 : cin), we(NT, max(a.m, 1)),
+      wz(NT, cout);
   auto load = [&](int t, int buf, bool zrow) {
     size_t p0;
     int np, x0;
     place(t, p0, np, x0);
     float* A = As + buf * PT * ap;
     const float* src = a.in + p0 * cin;
-    if ((cin & 3) == 0) {
-      const int q = cin >> 2;
-      for (int j = threadIdx.x; j < np * q; j += kPwThreads) {
-        const int p = j / q;
-        cpa16(A + p * ap + 4 * (j - p * q), src + 4 * j);
-      }
+    if (quad) {
+      for (Walk w = wa; w.r < np; w.next()) cpa16(A + w.r * ap + 4 * w.c, src + w.r * cin + 4 * w.c);
     } else {
-      for (int j = threadIdx.x; j < np * cin; j += kPwThreads) {
-        const int p = j / cin;
-        cpa4(A + p * ap + (j - p * cin), src + j);
-      }
+      for (Walk w = wa; w.r < np; w.next()) cpa4(A + w.r * ap + w.c, src + w.r * cin + w.c);
     }
     if (m2) {
-      for (int j = threadIdx.x; j < np * a.m; j += kPwThreads) {
-        const int p = j / a.m, c = j - p * a.m;
-        cpa8(A + p * ap + cin4 + 2 * c, a.ex + (size_t)(x0 + p) * a.ep + 2 * c);
-      }
+      for (Walk w = we; w.r < np; w.next())
+        cpa8(A + w.r * ap + cin4 + 2 * w.c, a.ex + (x0 + w.r) * a.ep + 2 * w.c);
       if (zrow) {
         const int row = t / a.tpr;
         float* Z = Zs + (row & 1) * OP * zp;
         const float* zr = reinterpret_cast<const float*>(a.z + (size_t)row * a.m * cout);
-        for (int j = threadIdx.x; j < a.m * cout; j += kPwThreads) {
-          const int kx = j / cout, o = j - kx * cout;
-          cpa8(Z + ((o & 3) * G + (o >> 2)) * zp + 2 * kx, zr + 2 * j);
-        }
+        for (Walk w = wz; w.r < a.m; w.next())
+          cpa8(Z + ((w.c & 3) * G + (w.c >> 2)) * zp + 2 * w.r, zr + 2 * (w.r * cout + w.c));
       }
     }
   };
@@ -371,19 +421,14 @@ __global__ void __launch_bounds__(kPwThreads, kPwCtas) k_tr_pw(const PwArgs a) {
     cpa_wait<1>();
     float* A = As + buf * PT * ap;
     if (a.in_act) {  // each thread the elements it copied
-      if ((cin & 3) == 0) {
-        const int q = cin >> 2;
-        for (int j = threadIdx.x; j < np * q; j += kPwThreads) {
-          const int p = j / q;
-          float4* e = reinterpret_cast<float4*>(A + p * ap + 4 * (j - p * q));
-          const float4 v = *e;
-          *e = make_float4(tr_act(v.x, a.act), tr_act(v.y, a.act), tr_act(v.z, a.act),
-                           tr_act(v.w, a.act));
+      if (quad) {
+        for (Walk w = wa; w.r < np; w.next()) {
+          float4* e = reinterpret_cast<float4*>(A + w.r * ap + 4 * w.c);
+          *e = tr_act4(*e, a.act);
         }
       } else {
-        for (int j = threadIdx.x; j < np * cin; j += kPwThreads) {
-          const int p = j / cin;
-          float* e = A + p * ap + (j - p * cin);
+        for (Walk w = wa; w.r < np; w.next()) {
+          float* e = A + w.r * ap + w.c;
           *e = tr_act(*e, a.act);
         }
       }
@@ -395,21 +440,36 @@ __global__ void __launch_bounds__(kPwThreads, kPwCtas) k_tr_pw(const PwArgs a) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
     auto sums = [&](const float* ar, const float* br, int bp, int n) {
-#pragma unroll 1
-      for (int k = 0; k < n; k += 4) {
+      const float *pa[PPT], *pb[4];  // running pointers: no address arithmetic but their steps
+#pragma unroll
+      for (int i = 0; i < PPT; ++i) pa[i] = ar + i * NPG * ap;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) pb[j] = br + j * G * bp;
+      auto term4 = [&](int at) {
         float4 b[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(br + j * G * bp + k);
+        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(pb[j] + at);
 #pragma unroll
         for (int i = 0; i < PPT; ++i) {
-          const float4 v = *reinterpret_cast<const float4*>(ar + i * NPG * ap + k);
+          const float4 v = *reinterpret_cast<const float4*>(pa[i] + at);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             acc[i][j] = __ffma2_rn(make_float2(v.x, v.y), make_float2(b[j].x, b[j].y), acc[i][j]);
             acc[i][j] = __ffma2_rn(make_float2(v.z, v.w), make_float2(b[j].z, b[j].w), acc[i][j]);
           }
         }
+      };
+      int k = 0;
+#pragma unroll 1
+      for (; k + 8 <= n; k += 8) {
+        term4(0);
+        term4(4);
+#pragma unroll
+        for (int i = 0; i < PPT; ++i) pa[i] += 8;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) pb[j] += 8;
       }
+      if (k < n) term4(0);
     };
     sums(A + pg * ap, Ws + og * wp, wp, cin4);
     if (m2) sums(A + pg * ap + cin4, Zs + ((t / a.tpr) & 1) * OP * zp + og * zp, zp, m24);
@@ -428,26 +488,54 @@ __global__ void __launch_bounds__(kPwThreads, kPwCtas) k_tr_pw(const PwArgs a) {
 #pragma unroll
           for (int j = 0; j < 4; ++j)
             if (og * 4 + j < cout) a.out[(b * cout + og * 4 + j) * a.hw + q] = v[j];
-        } else if ((cout & 3) == 0) {
-          if (a.pre) *reinterpret_cast<float4*>(a.pre + at) = make_float4(v[0], v[1], v[2], v[3]);
-          if (a.dz) {
-            const float4 d = *reinterpret_cast<const float4*>(a.dz + at);
-            v[0] *= tr_dact(d.x, a.act);
-            v[1] *= tr_dact(d.y, a.act);
-            v[2] *= tr_dact(d.z, a.act);
-            v[3] *= tr_dact(d.w, a.act);
-          } else if (a.out_act) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] = tr_act(v[j], a.act);
-          }
-          *reinterpret_cast<float4*>(a.out + at) = make_float4(v[0], v[1], v[2], v[3]);
         } else {
+          // derivative of the activation (pre) or of the one whose argument dz holds, and value
+          const bool quad_out = (cout & 3) == 0;
+          float2 w0 = make_float2(v[0], v[1]), w1 = make_float2(v[2], v[3]);
+          float2 f0 = w0, f1 = w1;
+          if (a.dz || a.d) {
+            float q[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            const float* from = (a.d ? a.d : a.dz) + at;
+            if (quad_out) {
+              const float4 q4 = *reinterpret_cast<const float4*>(from);
+              q[0] = q4.x;
+              q[1] = q4.y;
+              q[2] = q4.z;
+              q[3] = q4.w;
+            } else {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (og * 4 + j >= cout) continue;
-            if (a.pre) a.pre[at + j] = v[j];
-            a.out[at + j] = a.dz ? v[j] * tr_dact(a.dz[at + j], a.act)
-                                 : (a.out_act ? tr_act(v[j], a.act) : v[j]);
+              for (int j = 0; j < 4; ++j)
+                if (og * 4 + j < cout) q[j] = from[j];
+            }
+            float2 q0 = make_float2(q[0], q[1]), q1 = make_float2(q[2], q[3]);
+            if (!a.d) {
+              q0 = tr_dact2(q0, a.act);
+              q1 = tr_dact2(q1, a.act);
+            }
+            w0 = __fmul2_rn(w0, q0);
+            w1 = __fmul2_rn(w1, q1);
+          } else if (a.out_act) {
+            if (a.act == FNO_ACT_GELU) {
+              tr_gelu2(f0, &w0, &f0);
+              tr_gelu2(f1, &w1, &f1);
+            } else {
+              w0 = tr_act2(f0, a.act);
+              w1 = tr_act2(f1, a.act);
+              f0 = tr_dact2(f0, a.act);
+              f1 = tr_dact2(f1, a.act);
+            }
+          }
+          if (quad_out) {
+            if (a.pre) *reinterpret_cast<float4*>(a.pre + at) = make_float4(f0.x, f0.y, f1.x, f1.y);
+            *reinterpret_cast<float4*>(a.out + at) = make_float4(w0.x, w0.y, w1.x, w1.y);
+          } else {
+            const float f[4] = {f0.x, f0.y, f1.x, f1.y}, w[4] = {w0.x, w0.y, w1.x, w1.y};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              if (og * 4 + j >= cout) continue;
+              if (a.pre) a.pre[at + j] = f[j];
+              a.out[at + j] = w[j];
+            }
           }
         }
       }
@@ -467,18 +555,12 @@ struct WgArgs {
   size_t P;
   int cout, cin, in_act, act;
 };
-__device__ __forceinline__ void wg_load(const float* src, int n, int c, int pitch, float* dst) {
+__device__ __forceinline__ void wg_load(const float* src, int n, int c, int pitch, float* dst,
+                                        const Walk& from) {
   if ((c & 3) == 0) {
-    const int q = c >> 2;
-    for (int j = threadIdx.x; j < n * q; j += kWgThreads) {
-      const int p = j / q;
-      cpa16(dst + p * pitch + 4 * (j - p * q), src + 4 * j);
-    }
+    for (Walk w = from; w.r < n; w.next()) cpa16(dst + w.r * pitch + 4 * w.c, src + w.r * c + 4 * w.c);
   } else {
-    for (int j = threadIdx.x; j < n * c; j += kWgThreads) {
-      const int p = j / c;
-      cpa4(dst + p * pitch + (j - p * c), src + j);
-    }
+    for (Walk w = from; w.r < n; w.next()) cpa4(dst + w.r * pitch + w.c, src + w.r * c + w.c);
   }
 }
 __global__ void __launch_bounds__(kWgThreads, 2) k_tr_wgrad(const WgArgs a) {
@@ -491,15 +573,18 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_tr_wgrad(const WgArgs a) {
   const int og = tg / nti, ig = tg - og * nti;
   const int nbs = kWgThreads / dp, bo = threadIdx.x % dp, bs = threadIdx.x / dp;  // bias sums
   const int npairs = a.cout * (a.cin + 1);
+  const int sd = groups * dp, si = groups * ip;  // steps of a group's pixels
   for (int j = threadIdx.x; j < 2 * stage; j += kWgThreads) sm[j] = 0.0f;  // pads stay 0
   __syncthreads();
   const size_t tiles = (a.P + kWgTile - 1) / kWgTile;
   const size_t ta = tiles * blockIdx.x / gridDim.x, tb = tiles * (blockIdx.x + 1) / gridDim.x;
+  const Walk wd(kWgThreads, (a.cout & 3) ? a.cout : a.cout >> 2),
+      wi(kWgThreads, (a.cin & 3) ? a.cin : a.cin >> 2);
   auto load = [&](size_t t, float* st) {
     const size_t p0 = t * kWgTile;
     const int n = (int)min((size_t)kWgTile, a.P - p0);
-    wg_load(a.dz + p0 * a.cout, n, a.cout, dp, st);
-    wg_load(a.in + p0 * a.cin, n, a.cin, ip, st + kWgTile * dp);
+    wg_load(a.dz + p0 * a.cout, n, a.cout, dp, st, wd);
+    wg_load(a.in + p0 * a.cin, n, a.cin, ip, st + kWgTile * dp, wi);
   };
   float2 acc[8][4];
   float db = 0.0f;
@@ -518,18 +603,25 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_tr_wgrad(const WgArgs a) {
     const int n = (int)min((size_t)kWgTile, a.P - t * kWgTile);
     float* is = st + kWgTile * dp;
     if (a.in_act) {
-      for (int j = threadIdx.x; j < n * ip; j += kWgThreads) is[j] = tr_act(is[j], a.act);
+      for (int j = threadIdx.x; j < n * ip / 4; j += kWgThreads) {
+        float4* e = reinterpret_cast<float4*>(is) + j;
+        *e = tr_act4(*e, a.act);
+      }
       __syncthreads();
     }
     if (g < groups) {
+      const float *pd = st + g * dp + og * 4, *pe = pd + nto * 4;
+      const float *pv = is + g * ip + ig * 4, *pw = pv + nti * 4;
 #pragma unroll 2
       for (int p = g; p < n; p += groups) {
-        const float* d = st + p * dp + og * 4;
-        const float* v = is + p * ip + ig * 4;
-        const float4 d0 = *reinterpret_cast<const float4*>(d);
-        const float4 d1 = *reinterpret_cast<const float4*>(d + nto * 4);
-        const float4 v0 = *reinterpret_cast<const float4*>(v);
-        const float4 v1 = *reinterpret_cast<const float4*>(v + nti * 4);
+        const float4 d0 = *reinterpret_cast<const float4*>(pd);
+        const float4 d1 = *reinterpret_cast<const float4*>(pe);
+        const float4 v0 = *reinterpret_cast<const float4*>(pv);
+        const float4 v1 = *reinterpret_cast<const float4*>(pw);
+        pd += sd;
+        pe += sd;
+        pv += si;
+        pw += si;
         const float dd[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
         const float2 vv[4] = {make_float2(v0.x, v0.y), make_float2(v0.z, v0.w),
                               make_float2(v1.x, v1.y), make_float2(v1.z, v1.w)};
@@ -619,25 +711,21 @@ __global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f
   const size_t row0 = (size_t)blockIdx.x * rpb;
   const int nr = (int)min((size_t)rpb, rows - row0);
   const int nthr = blockDim.x;
+  const bool quad = (C & 3) == 0;
+  const Walk wf(nthr, quad ? C >> 2 : C);
   auto load = [&](int x0, float* st) {
     const int n = min(kDftX, W - x0);
     for (int r = 0; r < nr; ++r) {
       const float* src = f + ((row0 + r) * W + x0) * C;
-      if ((C & 3) == 0) {
-        const int q = C >> 2;
-        for (int j = threadIdx.x; j < n * q; j += nthr) {
-          const int x = j / q;
-          cpa16(st + x * kDftM + r * cp + 4 * (j - x * q), src + 4 * j);
-        }
+      float* d = st + r * cp;
+      if (quad) {
+        for (Walk w = wf; w.r < n; w.next()) cpa16(d + w.r * kDftM + 4 * w.c, src + w.r * C + 4 * w.c);
       } else {
-        for (int j = threadIdx.x; j < n * C; j += nthr) {
-          const int x = j / C;
-          cpa4(st + x * kDftM + r * cp + (j - x * C), src + j);
-        }
+        for (Walk w = wf; w.r < n; w.next()) cpa4(d + w.r * kDftM + w.c, src + w.r * C + w.c);
       }
     }
     float* es = st + kDftX * kDftM;
-    for (int j = threadIdx.x; j < n * (ep >> 2); j += nthr) cpa16(es + 4 * j, ex + (size_t)x0 * ep + 4 * j);
+    for (int j = threadIdx.x; j < n * (ep >> 2); j += nthr) cpa16(es + 4 * j, ex + x0 * ep + 4 * j);
   };
   float2 acc[4][NP];
 #pragma unroll
@@ -655,16 +743,19 @@ __global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f
     const float* st = sm + it * stage;
     const float* es = st + kDftX * kDftM + kg * 2 * NP;
     const int n = min(kDftX, W - x0);
+    const float *pv = st + sl * kDftM + 4 * lane, *pe = es + sl * ep;
 #pragma unroll 2
     for (int x = sl; x < n; x += ks) {
-      const float4 v = *reinterpret_cast<const float4*>(st + x * kDftM + 4 * lane);
+      const float4 v = *reinterpret_cast<const float4*>(pv);
       const float2 d[4] = {dup2(v.x), dup2(v.y), dup2(v.z), dup2(v.w)};
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
-        const float2 e = *reinterpret_cast<const float2*>(es + x * ep + 2 * k);
+        const float2 e = *reinterpret_cast<const float2*>(pe + 2 * k);
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[j][k] = __ffma2_rn(d[j], e, acc[j][k]);
       }
+      pv += ks * kDftM;
+      pe += ks * ep;
     }
     __syncthreads();
   }
@@ -904,36 +995,36 @@ struct TrCtx {
 
 // A row pitch of at least n floats: an odd number of 16-byte units.
 int odd_pitch(int n) { return 4 * (((n + 3) / 4) | 1); }
-constexpr int pw_tile(int op) { return op == 64 ? 64 : 128; }
+constexpr size_t kPwSmemMax = 227u << 10;
 struct PwSmem {
   int ap, wp, zp;
   size_t bytes;
 };
-PwSmem pw_smem(int op, int cin, int m) {
+PwSmem pw_smem(int op, int pt, int cin, int m) {
   PwSmem r;
   r.ap = odd_pitch((cin + 3) / 4 * 4 + 2 * m);
   r.wp = odd_pitch(cin);
   r.zp = m ? odd_pitch(2 * m) : 0;
-  r.bytes = sizeof(float) * ((size_t)2 * pw_tile(op) * r.ap + (size_t)op * (r.wp + 2 * r.zp));
+  r.bytes = sizeof(float) * ((size_t)2 * pt * r.ap + (size_t)op * (r.wp + 2 * r.zp));
   return r;
 }
-template <int OP>
+template <int OP, int PT, int NT>
 int pw_run(const TrCtx& x, PwArgs a) {
-  constexpr int PT = pw_tile(OP);
-  const PwSmem sm = pw_smem(OP, a.cin, a.z ? a.m : 0);
+  const PwSmem sm = pw_smem(OP, PT, a.cin, a.z ? a.m : 0);
   a.ap = sm.ap;
   a.wp = sm.wp;
   a.zp = sm.zp;
   a.tpr = (a.W + PT - 1) / PT;
   a.ntiles = a.z ? x.B * x.H * a.tpr : (int)((a.P + PT - 1) / PT);
-  const int ctas = std::max(1, std::min<int>(kPwCtas, (int)((227 << 10) / (sm.bytes + 1024))));
-  k_tr_pw<OP, PT><<<std::min(a.ntiles, ctas * kTrSms), kPwThreads, sm.bytes, x.st>>>(a);
+  const int ctas = std::max(1, std::min<int>(pw_ctas(NT), (int)((227 << 10) / (sm.bytes + 1024))));
+  k_tr_pw<OP, PT, NT><<<std::min(a.ntiles, ctas * kTrSms), NT, sm.bytes, x.st>>>(a);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
 // What one pointwise launch does besides its layer (PwArgs).
 struct PwOpt {
   const float2* z = nullptr;
+  const float* d = nullptr;
   const float* dz = nullptr;
   float* pre = nullptr;
   int in_act = 0, out_act = 0, planar = 0;
@@ -946,6 +1037,7 @@ int pw(const TrCtx& x, const float* in, int cin, const float* w, int trans, cons
   a.bias = bias;
   a.z = o.z;
   a.ex = reinterpret_cast<const float*>(x.ws + x.pl.ex);
+  a.d = o.d;
   a.dz = o.dz;
   a.pre = o.pre;
   a.out = out;
@@ -961,8 +1053,15 @@ int pw(const TrCtx& x, const float* in, int cin, const float* w, int trans, cons
   a.W = x.W;
   a.m = x.c->modes;
   a.ep = x.pl.ep;
-  // output columns of a block: the smallest tile that holds them
-  return cout > 32 ? pw_run<64>(x, a) : (cout > 16 ? pw_run<32>(x, a) : pw_run<16>(x, a));
+  // Output columns of a block: the smallest tile that holds them.  64 columns: 256 pixels,
+  // eight a thread (fewest shared loads a sum), when the stages fit and rows fill the tile.
+  if (cout > 32) {
+    if (pw_smem(64, 256, a.cin, a.z ? a.m : 0).bytes <= kPwSmemMax &&
+        (a.z ? (a.W + 255) / 256 * 256 <= a.W + a.W / 4 : a.P >= (size_t)256 * kTrSms))
+      return pw_run<64, 256, 512>(x, a);
+    return pw_run<64, 64, 256>(x, a);
+  }
+  return cout > 16 ? pw_run<32, 128, 256>(x, a) : pw_run<16, 128, 256>(x, a);
 }
 
 size_t wg_smem(int cout, int cin) {
@@ -1021,9 +1120,10 @@ cudaError_t smem_limit(K k, size_t bytes) {
 int set_smem_limits() {
   static bool done = false;
   if (done) return LBM_OK;
-  LBM_CHECK_CUDA(smem_limit(k_tr_pw<64, pw_tile(64)>, pw_smem(64, 64, kTrModesMax).bytes));
-  LBM_CHECK_CUDA(smem_limit(k_tr_pw<32, pw_tile(32)>, pw_smem(32, 64, kTrModesMax).bytes));
-  LBM_CHECK_CUDA(smem_limit(k_tr_pw<16, pw_tile(16)>, pw_smem(16, 64, kTrModesMax).bytes));
+  LBM_CHECK_CUDA(smem_limit(k_tr_pw<64, 256, 512>, kPwSmemMax));
+  LBM_CHECK_CUDA(smem_limit(k_tr_pw<64, 64, 256>, pw_smem(64, 64, 64, kTrModesMax).bytes));
+  LBM_CHECK_CUDA(smem_limit(k_tr_pw<32, 128, 256>, pw_smem(32, 128, 64, kTrModesMax).bytes));
+  LBM_CHECK_CUDA(smem_limit(k_tr_pw<16, 128, 256>, pw_smem(16, 128, 64, kTrModesMax).bytes));
   LBM_CHECK_CUDA(smem_limit(k_tr_wgrad, wg_smem(64, 64)));
   LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<4>, dft_x_smem(64, 8, 4)));
   LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<6>, dft_x_smem(72, 8, 5)));
@@ -1186,7 +1286,8 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
     const int fan = (l == 0) ? C : S;
     LBM_TRY(wgrad(x, g, S, lin, fan, l == 0 ? 0 : 1, dp + o.dec_w[l], dp + o.dec_b[l]));
     float* gn = (g == ta) ? tb : ta;
-    opt.dz = (l == 0) ? zpre(c.layers - 1) : hdpre(l - 1);
+    opt.d = (l == 0) ? zpre(c.layers - 1) : nullptr;
+    opt.dz = (l == 0) ? nullptr : hdpre(l - 1);
     LBM_TRY(pw(x, g, S, p + o.dec_w[l], 1, nullptr, fan, gn, opt));
     g = gn;
   }
@@ -1204,13 +1305,14 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
     float* gn = (g == ta) ? tb : ta;
     PwOpt lo;
     lo.z = reinterpret_cast<const float2*>(x.ws + pl.z);
-    lo.dz = n > 0 ? zpre(n - 1) : nullptr;
+    lo.d = n > 0 ? zpre(n - 1) : nullptr;
     LBM_TRY(pw(x, g, C, p + o.w[n], 1, nullptr, C, gn, lo));
     g = gn;
   }
   // lifting network: g = dL/dtheta_0
   LBM_TRY(wgrad(x, g, C, h1pre, h, 1, dp + o.lift1_w, dp + o.lift1_b));
   float* gh = (g == ta) ? tb : ta;
+  opt.d = nullptr;
   opt.dz = h1pre;
   LBM_TRY(pw(x, g, C, p + o.lift1_w, 1, nullptr, h, gh, opt));
   LBM_TRY(wgrad(x, gh, h, xin, c.c_in + 2, 0, dp + o.lift0_w, dp + o.lift0_b));
