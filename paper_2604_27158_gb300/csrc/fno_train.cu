@@ -99,6 +99,7 @@ struct TrPlan {
   size_t xin, h1pre, theta, zpre, xh, hdpre, saved_floats;
   // workspace, in bytes
   size_t rt, x1, yh, dyh, z, ta, tb, part, ex, ey, ycl, ws_bytes;
+  size_t s, twx, twy;  // ReLU forward pass
   int wg_blocks;
   int np, ng, ep;  // x-DFT: kx pairs a thread, thread groups, floats a row of the table
 };
@@ -153,6 +154,11 @@ TrPlan tr_plan(const fno_config& c, int B, int H, int W) {
   t.ex = take((size_t)W * t.ep * sizeof(float));
   t.ey = take((size_t)H * 2 * m * sizeof(float4));
   t.ycl = take(P * c.c_out * sizeof(float));
+  if (c.activation == FNO_ACT_RELU) {
+    t.s = take(P * C * sizeof(float));
+    t.twx = take((size_t)W * sizeof(float2));
+    t.twy = take((size_t)H * sizeof(float2));
+  }
   t.ws_bytes = b;
   return t;
 }
@@ -844,6 +850,252 @@ __global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
   }
 }
 
+// ---- forward pass of ReLU networks -----------------------------------------------------------
+// ReLU's derivative jumps at 0.  Sums in another order move the pre-activations that lie within
+// rounding of 0 across it, and one pixel that changes sides changes a gradient, a sum over pixels
+// with random signs, by 1e-4 of its norm or more.  So that a ReLU network's gradients do not
+// depend on how its layers are tiled, its forward pass keeps one plain order: every sum runs
+// over its terms one after the other (the kernels below, one output a thread and term loop).  Its
+// backward pass, which takes the signs as saved, uses the tiled kernels.
+constexpr int kSqPix = 128;      // pixels a block of the pointwise kernel
+constexpr int kSqThreads = 256;
+constexpr int kSqAcc = 16;       // spectral accumulators a thread
+
+__global__ void k_sq_twiddle(float2* __restrict__ tw, int N) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < N) {
+    double s, c;
+    sincospi(2.0 * (double)t / (double)N, &s, &c);
+    tw[t] = make_float2((float)c, (float)s);
+  }
+}
+
+// Pointwise linear layer over kSqPix pixels per block:
+//   v[p][o] = add[p][o] + bias[o] + sum_i Wm(o, i) * A(in[p][i]),
+//   Wm(o, i) = trans ? w[i * cout + o] : w[o * cin + i],  A = sigma if in_act else identity;
+//   pre[p][o] = v (if pre != null);  out[p][o] = out_act ? sigma(v) : v.
+__global__ void __launch_bounds__(kSqPix) k_sq_pw(const float* __restrict__ in, int cin,
+                                                  const float* __restrict__ w, int trans,
+                                                  const float* __restrict__ bias,
+                                                  const float* __restrict__ add, int cout,
+                                                  float* __restrict__ pre, float* __restrict__ out,
+                                                  int in_act, int out_act, int act, size_t P) {
+  extern __shared__ float sm[];
+  float* ws = sm;                               // [cout][cin]
+  float* is = ws + cout * cin;                  // [kSqPix][cin + 1]
+  float* os = is + kSqPix * (cin + 1);          // [kSqPix][cout + 1]
+  const size_t p0 = (size_t)blockIdx.x * kSqPix;
+  const int np = (int)min((size_t)kSqPix, P - p0);
+  for (int j = threadIdx.x; j < cout * cin; j += kSqPix) {
+    const int o = j / cin, i = j - o * cin;
+    ws[j] = trans ? w[(size_t)i * cout + o] : w[j];
+  }
+  for (int j = threadIdx.x; j < np * cin; j += kSqPix) {
+    const int t = j / cin, i = j - t * cin;
+    const float v = in[p0 * cin + j];
+    is[t * (cin + 1) + i] = in_act ? tr_act(v, act) : v;
+  }
+  for (int j = threadIdx.x; j < np * cout; j += kSqPix) {
+    const int t = j / cout, o = j - t * cout;
+    os[t * (cout + 1) + o] = (add ? add[p0 * cout + j] : 0.0f) + (bias ? bias[o] : 0.0f);
+  }
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t < np) {
+    const float* ir = is + t * (cin + 1);
+    float* orow = os + t * (cout + 1);
+    for (int o = 0; o < cout; ++o) {
+      const float* wr = ws + o * cin;
+      float acc = 0.0f;
+      for (int i = 0; i < cin; ++i) acc = fmaf(wr[i], ir[i], acc);
+      orow[o] += acc;
+    }
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < np * cout; j += kSqPix) {
+    const int tt = j / cout, o = j - tt * cout;
+    const float v = os[tt * (cout + 1) + o];
+    if (pre) pre[p0 * cout + j] = v;
+    out[p0 * cout + j] = out_act ? tr_act(v, act) : v;
+  }
+}
+
+// Forward x-DFT of each row: X1[row][kx][c] = sum_x f[row][x][c] e^{-2 pi i kx x / W}.
+__global__ void __launch_bounds__(kSqThreads) k_sq_dft_x(const float* __restrict__ f,
+                                                           float2* __restrict__ x1,
+                                                           const float2* __restrict__ twx,
+                                                           int W, int C, int m) {
+  extern __shared__ float sm[];
+  float2* tw = reinterpret_cast<float2*>(sm);  // W
+  float* tile = sm + 2 * W;                     // [32][C]
+  const size_t row = blockIdx.x;
+  for (int t = threadIdx.x; t < W; t += kSqThreads) tw[t] = twx[t];
+  const int G = kSqThreads / C;
+  const int c = threadIdx.x % C, g = threadIdx.x / C;
+  float2 acc[kSqAcc];
+#pragma unroll
+  for (int k = 0; k < kSqAcc; ++k) acc[k] = make_float2(0.f, 0.f);
+  for (int x0 = 0; x0 < W; x0 += 32) {
+    const int nx = min(32, W - x0);
+    __syncthreads();
+    for (int j = threadIdx.x; j < nx * C; j += kSqThreads)
+      tile[j] = f[(row * W + x0) * C + j];
+    __syncthreads();
+    if (g < G) {
+#pragma unroll
+      for (int k = 0; k < kSqAcc; ++k) {
+        const int kx = g + k * G;
+        if (kx < m) {
+          int idx = (kx * x0) % W;  // phase index (kx x) mod W, advanced by kx per x
+          for (int xx = 0; xx < nx; ++xx) {
+            const float2 e = tw[idx];
+            const float v = tile[xx * C + c];
+            acc[k].x = fmaf(v, e.x, acc[k].x);
+            acc[k].y = fmaf(-v, e.y, acc[k].y);
+            idx += kx;
+            if (idx >= W) idx -= W;
+          }
+        }
+      }
+    }
+  }
+  if (g < G) {
+#pragma unroll
+    for (int k = 0; k < kSqAcc; ++k) {
+      const int kx = g + k * G;
+      if (kx < m) x1[(row * m + kx) * C + c] = acc[k];
+    }
+  }
+}
+
+// Forward y-DFT over the kept rows: Xh[b][a][kx][c] = scale(kx) sum_y X1[b][y][kx][c]
+// e^{-2 pi i ky(a) y / H}, ky(a) = a (a < m) or H - 2m + a; scale = 1, or c_kx / (H W)
+// for the adjoint of the real inverse transform.
+__global__ void __launch_bounds__(kSqThreads) k_sq_dft_y(const float2* __restrict__ x1,
+                                                           float2* __restrict__ xh,
+                                                           const float2* __restrict__ twy,
+                                                           int H, int W, int C, int m,
+                                                           int adjoint_scale) {
+  extern __shared__ float sm[];
+  float2* tw = reinterpret_cast<float2*>(sm);  // H
+  float2* tile = tw + H;                        // [32][C]
+  const int b = blockIdx.x / m, kx = blockIdx.x % m;
+  for (int t = threadIdx.x; t < H; t += kSqThreads) tw[t] = twy[t];
+  const int G = kSqThreads / C;
+  const int c = threadIdx.x % C, g = threadIdx.x / C;
+  float2 acc[kSqAcc];
+#pragma unroll
+  for (int k = 0; k < kSqAcc; ++k) acc[k] = make_float2(0.f, 0.f);
+  for (int y0 = 0; y0 < H; y0 += 32) {
+    const int ny = min(32, H - y0);
+    __syncthreads();
+    for (int j = threadIdx.x; j < ny * C; j += kSqThreads) {
+      const int yy = j / C, cc = j - yy * C;
+      tile[j] = x1[(((size_t)b * H + y0 + yy) * m + kx) * C + cc];
+    }
+    __syncthreads();
+    if (g < G) {
+#pragma unroll
+      for (int k = 0; k < kSqAcc; ++k) {
+        const int a = g + k * G;
+        if (a < 2 * m) {
+          const int ky = a < m ? a : H - 2 * m + a;
+          int idx = (int)(((long long)ky * y0) % H);  // (ky y) mod H, advanced by ky per y
+          for (int yy = 0; yy < ny; ++yy) {
+            const float2 e = tw[idx];  // e^{+i}: use conj
+            idx += ky;
+            if (idx >= H) idx -= H;
+            const float2 v = tile[yy * C + c];
+            // v * conj(e)
+            acc[k].x = fmaf(v.x, e.x, fmaf(v.y, e.y, acc[k].x));
+            acc[k].y = fmaf(v.y, e.x, fmaf(-v.x, e.y, acc[k].y));
+          }
+        }
+      }
+    }
+  }
+  const float sc = adjoint_scale ? (kx == 0 ? 1.0f : 2.0f) / ((float)H * (float)W) : 1.0f;
+  if (g < G) {
+#pragma unroll
+    for (int k = 0; k < kSqAcc; ++k) {
+      const int a = g + k * G;
+      if (a < 2 * m)
+        xh[(((size_t)b * 2 * m + a) * m + kx) * C + c] = make_float2(acc[k].x * sc, acc[k].y * sc);
+    }
+  }
+}
+
+// Inverse y-DFT: Z[b][y][kx][c] = sum_a Yh[b][a][kx][c] e^{+2 pi i ky(a) y / H}.
+__global__ void __launch_bounds__(kSqThreads) k_sq_inv_y(const float2* __restrict__ yh,
+                                                           float2* __restrict__ z,
+                                                           const float2* __restrict__ twy,
+                                                           int H, int C, int m) {
+  extern __shared__ float sm[];
+  float2* tw = reinterpret_cast<float2*>(sm);  // H
+  float2* col = tw + H;                         // [2m][C]
+  const int b = blockIdx.x / m, kx = blockIdx.x % m;
+  for (int t = threadIdx.x; t < H; t += kSqThreads) tw[t] = twy[t];
+  for (int j = threadIdx.x; j < 2 * m * C; j += kSqThreads) {
+    const int a = j / C, c = j - a * C;
+    col[j] = yh[(((size_t)b * 2 * m + a) * m + kx) * C + c];
+  }
+  __syncthreads();
+  const int G = kSqThreads / C;
+  const int c = threadIdx.x % C, g = threadIdx.x / C;
+  if (g >= G) return;
+  for (int y = g; y < H; y += G) {
+    float re = 0.f, im = 0.f;
+    int idx = 0;  // (ky y) mod H for ky = 0 .. m-1, then H-m .. H-1
+    for (int a = 0; a < 2 * m; ++a) {
+      if (a == m) idx = (int)(((long long)(H - m) * y) % H);
+      const float2 e = tw[idx];
+      idx += y;
+      if (idx >= H) idx -= H;
+      const float2 v = col[a * C + c];
+      re = fmaf(v.x, e.x, fmaf(-v.y, e.y, re));
+      im = fmaf(v.x, e.y, fmaf(v.y, e.x, im));
+    }
+    z[(((size_t)b * H + y) * m + kx) * C + c] = make_float2(re, im);
+  }
+}
+
+// Inverse x-DFT with real output: S[row][x][c] = scale sum_kx w(kx) Re(Z[row][kx][c]
+// e^{+2 pi i kx x / W}); w(kx) = c_kx (forward) or 1 (adjoint of the forward DFT).
+__global__ void __launch_bounds__(kSqThreads) k_sq_inv_x(const float2* __restrict__ z,
+                                                           float* __restrict__ s,
+                                                           const float2* __restrict__ twx,
+                                                           int W, int C, int m, float scale,
+                                                           int hermitian) {
+  extern __shared__ float sm[];
+  float2* tw = reinterpret_cast<float2*>(sm);  // W
+  float2* zr = tw + W;                          // [m][C]
+  const size_t row = blockIdx.x;
+  for (int t = threadIdx.x; t < W; t += kSqThreads) tw[t] = twx[t];
+  for (int j = threadIdx.x; j < m * C; j += kSqThreads) {
+    const int kx = j / C;
+    float2 v = z[row * m * C + j];
+    const float wk = (hermitian && kx > 0) ? 2.0f * scale : scale;
+    zr[j] = make_float2(v.x * wk, v.y * wk);
+  }
+  __syncthreads();
+  const int G = kSqThreads / C;
+  const int c = threadIdx.x % C, g = threadIdx.x / C;
+  if (g >= G) return;
+  for (int x = g; x < W; x += G) {
+    float acc = 0.f;
+    int idx = 0;  // (kx x) mod W
+    for (int kx = 0; kx < m; ++kx) {
+      const float2 e = tw[idx];
+      idx += x;
+      if (idx >= W) idx -= W;
+      const float2 v = zr[kx * C + c];
+      acc = fmaf(v.x, e.x, fmaf(-v.y, e.y, acc));
+    }
+    s[(row * W + x) * C + c] = acc;
+  }
+}
+
+// ---- both -------------------------------------------------------------------------------------
 // Per-mode channel mixing and its two adjoints (modes = 2 m m, Rt[mode][i][o]).
 __global__ void k_tr_mix(const float2* __restrict__ xh, const float2* __restrict__ rt,
                          float2* __restrict__ yh, int B, int C, int modes) {
@@ -957,6 +1209,17 @@ __global__ void __launch_bounds__(256) k_tr_inv_y(const float2* __restrict__ yh,
   }
 }
 
+__global__ void k_sq_cl_to_nchw(const float* __restrict__ cl, float* __restrict__ out, int B,
+                                int H, int W, int C) {
+  const size_t n = (size_t)B * C * H * W;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const size_t hw = (size_t)H * W;
+  const int b = (int)(t / (C * hw));
+  const int c = (int)((t / hw) % C);
+  const size_t q = t % hw;
+  out[t] = cl[((size_t)b * hw + q) * C + c];
+}
 // planar -> channels-last for the gradient of the output
 __global__ void k_tr_nchw_to_cl(const float* __restrict__ in, float* __restrict__ cl, int B, int H,
                                 int W, int C) {
@@ -1113,6 +1376,96 @@ int spectral_inv(const TrCtx& x, const float2* coef, float scale, int hermitian)
   return LBM_OK;
 }
 
+// The ReLU forward pass.
+size_t sq_pw_smem(int cin, int cout) {
+  return sizeof(float) * ((size_t)cout * cin + (size_t)kSqPix * (cin + 1) + (size_t)kSqPix * (cout + 1));
+}
+
+int sq_pw(const TrCtx& x, const float* in, int cin, const float* w, int trans, const float* bias,
+       const float* add, int cout, float* pre, float* out, int in_act, int out_act) {
+  const size_t smem = sq_pw_smem(cin, cout);
+  k_sq_pw<<<nb(x.pl.P, kSqPix), kSqPix, smem, x.st>>>(in, cin, w, trans, bias, add, cout, pre, out,
+                                                      in_act, out_act, x.c->activation, x.pl.P);
+  LBM_CHECK_LAUNCH();
+  return LBM_OK;
+}
+
+// X (or the adjoint-scaled dY) of a field: forward x-DFT then y-DFT over the kept rows.
+int sq_spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_scale) {
+  const int C = x.c->width, m = x.c->modes;
+  float2* x1 = reinterpret_cast<float2*>(x.ws + x.pl.x1);
+  const float2* twx = reinterpret_cast<const float2*>(x.ws + x.pl.twx);
+  const float2* twy = reinterpret_cast<const float2*>(x.ws + x.pl.twy);
+  k_sq_dft_x<<<x.B * x.H, kSqThreads, (2 * x.W + 32 * C) * sizeof(float), x.st>>>(f, x1, twx, x.W,
+                                                                                    C, m);
+  LBM_CHECK_LAUNCH();
+  k_sq_dft_y<<<x.B * m, kSqThreads, (x.H + 32 * C) * sizeof(float2), x.st>>>(
+      x1, out, twy, x.H, x.W, C, m, adjoint_scale);
+  LBM_CHECK_LAUNCH();
+  return LBM_OK;
+}
+
+// Real field from kept coefficients: inverse y-DFT then inverse x-DFT.
+int sq_spectral_inv(const TrCtx& x, const float2* coef, float* s, float scale, int hermitian) {
+  const int C = x.c->width, m = x.c->modes;
+  float2* z = reinterpret_cast<float2*>(x.ws + x.pl.z);
+  const float2* twx = reinterpret_cast<const float2*>(x.ws + x.pl.twx);
+  const float2* twy = reinterpret_cast<const float2*>(x.ws + x.pl.twy);
+  k_sq_inv_y<<<x.B * m, kSqThreads, (x.H + 2 * m * C) * sizeof(float2), x.st>>>(coef, z, twy,
+                                                                                  x.H, C, m);
+  LBM_CHECK_LAUNCH();
+  k_sq_inv_x<<<x.B * x.H, kSqThreads, (x.W + m * C) * sizeof(float2), x.st>>>(z, s, twx, x.W, C, m,
+                                                                                scale, hermitian);
+  LBM_CHECK_LAUNCH();
+  return LBM_OK;
+}
+
+
+int sq_forward(const TrCtx& x, const float* params, const float* xin, float* saved, float* out_d) {
+  const fno_config& c = *x.c;
+  const TrPlan& pl = x.pl;
+  const TrOff& o = x.off;
+  const int B = x.B, C = c.width, h = C / 2, S = c.dec_size, m = c.modes;
+  const size_t P = pl.P, spec = (size_t)B * 2 * m * m * C;
+  float* ta = reinterpret_cast<float*>(x.ws + pl.ta);
+  float* tb = reinterpret_cast<float*>(x.ws + pl.tb);
+  float* s = reinterpret_cast<float*>(x.ws + pl.s);
+  float* ycl = reinterpret_cast<float*>(x.ws + pl.ycl);
+  float2* yh = reinterpret_cast<float2*>(x.ws + pl.yh);
+  const float2* rt = reinterpret_cast<const float2*>(x.ws + pl.rt);
+  const float* p = params;
+  auto theta = [&](int n) { return saved + pl.theta + (size_t)n * P * C; };
+  k_sq_twiddle<<<nb(x.W), 256, 0, x.st>>>(reinterpret_cast<float2*>(x.ws + pl.twx), x.W);
+  LBM_CHECK_LAUNCH();
+  k_sq_twiddle<<<nb(x.H), 256, 0, x.st>>>(reinterpret_cast<float2*>(x.ws + pl.twy), x.H);
+  LBM_CHECK_LAUNCH();
+  LBM_TRY(sq_pw(x, xin, c.c_in + 2, p + o.lift0_w, 0, p + o.lift0_b, nullptr, h, saved + pl.h1pre,
+                ta, 0, 1));
+  LBM_TRY(sq_pw(x, ta, h, p + o.lift1_w, 0, p + o.lift1_b, nullptr, C, nullptr, theta(0), 0, 0));
+  for (int n = 0; n < c.layers; ++n) {
+    float2* xh = reinterpret_cast<float2*>(saved + pl.xh) + (size_t)n * spec;
+    LBM_TRY(sq_spectral_fwd(x, theta(n), xh, 0));
+    k_tr_mix<<<nb(spec), 256, 0, x.st>>>(xh, rt + (size_t)n * 2 * m * m * C * C, yh, B, C, 2 * m * m);
+    LBM_CHECK_LAUNCH();
+    LBM_TRY(sq_spectral_inv(x, yh, s, 1.0f / ((float)x.H * (float)x.W), 1));
+    LBM_TRY(sq_pw(x, theta(n), C, p + o.w[n], 0, p + o.b[n], s, C, saved + pl.zpre + (size_t)n * P * C,
+                  theta(n + 1), 0, 1));
+  }
+  const float* hin = theta(c.layers);
+  int fan = C;
+  for (int l = 0; l < c.dec_layers; ++l) {
+    float* hout = (l % 2 == 0) ? ta : tb;
+    LBM_TRY(sq_pw(x, hin, fan, p + o.dec_w[l], 0, p + o.dec_b[l], nullptr, S,
+                  saved + pl.hdpre + (size_t)l * P * S, hout, 0, 1));
+    hin = hout;
+    fan = S;
+  }
+  LBM_TRY(sq_pw(x, hin, fan, p + o.out_w, 0, p + o.out_b, nullptr, c.c_out, nullptr, ycl, 0, 0));
+  k_sq_cl_to_nchw<<<nb(P * c.c_out), 256, 0, x.st>>>(ycl, out_d, B, x.H, x.W, c.c_out);
+  LBM_CHECK_LAUNCH();
+  return LBM_OK;
+}
+
 template <typename K>
 cudaError_t smem_limit(K k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -1130,6 +1483,16 @@ int set_smem_limits() {
   LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<7>, dft_x_smem(72, 8, 5)));
   LBM_CHECK_CUDA(smem_limit(k_tr_dft_x<8>, dft_x_smem(64, 8, 4)));
   LBM_CHECK_CUDA(smem_limit(k_tr_inv_y, inv_y_smem(kTrModesMax)));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_sq_pw, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sq_pw_smem(64, 64)));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_sq_dft_x, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)((2 * 2048 + 32 * 64) * sizeof(float))));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_sq_dft_y, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)((8192 + 32 * 64) * sizeof(float2))));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_sq_inv_y, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)((8192 + 2 * kTrModesMax * 64) * sizeof(float2))));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_sq_inv_x, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)((2048 + kTrModesMax * 64) * sizeof(float2))));
   done = true;
   return LBM_OK;
 }
@@ -1217,6 +1580,7 @@ int fno_train_forward(const fno_config* cfg_h, const float* params_d, const floa
 
   k_tr_xin<<<nb(P), 256, 0, x.st>>>(in_d, xin, B, H, W, c.c_in);
   LBM_CHECK_LAUNCH();
+  if (c.activation == FNO_ACT_RELU) return sq_forward(x, p, xin, saved_d, out_d);
   // hidden layers store their pre-activations only; the next layer applies sigma as it reads
   LBM_TRY(pw(x, xin, c.c_in + 2, p + o.lift0_w, 0, p + o.lift0_b, h, h1pre));
   PwOpt act_in;
@@ -1275,6 +1639,7 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
   k_tr_nchw_to_cl<<<nb(P * c.c_out), 256, 0, x.st>>>(dout_d, ycl, B, H, W, c.c_out);
   LBM_CHECK_LAUNCH();
   const int L = c.dec_layers;
+  const bool relu = c.activation == FNO_ACT_RELU;  // zpre holds z, not sigma'(z)
   // g: gradient with respect to the pre-activation of the layer at hand, in ta or tb
   LBM_TRY(wgrad(x, ycl, c.c_out, hdpre(L - 1), S, 1, dp + o.out_w, dp + o.out_b));
   PwOpt opt;
@@ -1286,8 +1651,8 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
     const int fan = (l == 0) ? C : S;
     LBM_TRY(wgrad(x, g, S, lin, fan, l == 0 ? 0 : 1, dp + o.dec_w[l], dp + o.dec_b[l]));
     float* gn = (g == ta) ? tb : ta;
-    opt.d = (l == 0) ? zpre(c.layers - 1) : nullptr;
-    opt.dz = (l == 0) ? nullptr : hdpre(l - 1);
+    opt.d = (l == 0 && !relu) ? zpre(c.layers - 1) : nullptr;
+    opt.dz = (l == 0) ? zpre(c.layers - 1) : hdpre(l - 1);
     LBM_TRY(pw(x, g, S, p + o.dec_w[l], 1, nullptr, fan, gn, opt));
     g = gn;
   }
@@ -1305,7 +1670,8 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
     float* gn = (g == ta) ? tb : ta;
     PwOpt lo;
     lo.z = reinterpret_cast<const float2*>(x.ws + pl.z);
-    lo.d = n > 0 ? zpre(n - 1) : nullptr;
+    lo.d = n > 0 && !relu ? zpre(n - 1) : nullptr;
+    lo.dz = n > 0 ? zpre(n - 1) : nullptr;
     LBM_TRY(pw(x, g, C, p + o.w[n], 1, nullptr, C, gn, lo));
     g = gn;
   }

@@ -23,6 +23,8 @@ struct Handle {
   bool persistent = false;     // lbm_step runs nsteps > 1 in one multi-step launch
   unsigned* bar_count = nullptr;  // grid-barrier counter of the multi-step launch
   int4* tiles_d[LBM_STEP_VARIANTS] = {};      // per-shape tile descriptors (workspace)
+  bool dense4 = false;  // every nx is a multiple of 4: dense and canonical rows are 16-byte
+                        // aligned whenever their buffers are
   struct SweepTask* sweep_d = nullptr;  // tasks of a multi-step pass (workspace)
   int sweep_ctas = 0;
   unsigned* status_d = nullptr;
@@ -49,6 +51,8 @@ int residual_step(Handle* h, double* out_h, int update_prev, cudaStream_t s);
 // f = f^eq(rho, u) (+ f^neq) of every grid into the current buffer (reinit.cu), one CTA
 // a tile of the step-kernel tile table with kReinitRows rows a tile.
 constexpr int kReinitRows = 6;
+// The chunk kernels (lbm_chunk.cuh) take the tile table of shape kChunkVariant (4 rows).
+constexpr int kChunkVariant = 1;
 int reinit_init(Handle* h);  // sets the kernel's shared-memory limit (once per handle)
 int reinit_launch(Handle* h, const int4* tiles, int ntiles, const float* rho_d,
                   const float* ux_d, const float* uy_d, int neq_mode, cudaStream_t s);
