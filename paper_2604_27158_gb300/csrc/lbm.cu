@@ -1203,6 +1203,7 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
   sweep_plan(h->gd, &sweep);
   h->sweep_d = reinterpret_cast<SweepTask*>(ws + wp.sweep_off);
   h->sweep_ctas = (int)(sweep.size() / kSweepWarps);
+  h->sweep = sweep_pays(h->gd);
   h->stats_h.assign((size_t)ngrids * R_COUNT, 0.0);
   h->u_max2 = (float)(u_max * u_max);
   cudaStream_t s = S(stream);
@@ -1263,7 +1264,7 @@ int lbm_step(lbm_handle* h, int nsteps, void* stream) {
     return LBM_OK;
   }
   int left = nsteps;
-  for (; left >= kSweepSteps; left -= kSweepSteps) {
+  for (; h->sweep && left >= kSweepSteps; left -= kSweepSteps) {
     LBM_TRY(sweep_launch(h, h->f[h->cur], h->f[h->cur ^ 1], s));
     h->cur ^= 1;
   }

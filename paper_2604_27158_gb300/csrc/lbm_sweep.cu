@@ -20,11 +20,11 @@
 // side, whose lanes compute but do not store (a level spoils one more column inwards).  Tasks
 // overlap in y the same way: a task of l rows computes l + 2 rows of level 1.
 //
-// Rounding.  The unforced collision runs on packed pairs with the operations of the
-// single-step kernel in the same order; the file is compiled without multiply-add
-// contraction; a body force takes the scalar code.  States are bitwise those of single steps.
+// Rounding.  The collision runs on packed pairs with the operations of the single-step kernel in
+// the same order; the file is compiled without multiply-add contraction.  States are bitwise
+// those of single steps.
 //
-// What bounds it (64 grids of 512 x 256): 57.8 us a step.  The pass moves 5.2 TB/s; issue
+// What bounds it (64 grids of 512 x 256): 58 us a step.  The pass moves 5.2 TB/s; issue
 // slots are 46% busy with the eleven warps a multiprocessor that the shared memory of the
 // kept rows allows, and their fixed-latency chains are what is left.  Measured and not kept:
 // two cells a lane and 24 warps (89 us: the per-lane work is not halved), the kept rows in
@@ -166,6 +166,39 @@ __device__ __forceinline__ void collide2(float om1, float2 drho, float2 rho, flo
   relax_pair2(g[6], g[8], a2, n2, b2, sub2(uy, ux), e2, om);
 }
 
+// The forced collision (Guo source) on two cells, in the order of collide().  Its products feed
+// sums; the assembler contracts a packed product and sum that are separate instructions, so the
+// sums here are multiply-adds with `one`, a 1 it cannot see (a run-time value).
+__device__ __forceinline__ void forced_pair2(float2& gi, float2& go, float w, float2 cu, float cf,
+                                             float2 drho, float2 rho, float2 usq, float2 om,
+                                             float2 sym_f, float guo, float2 one) {
+  auto add = [&](float2 a, float2 b) { return fma2(a, one, b); };
+  const float2 q = mul2(mul2(dup(4.5f), cu), cu);
+  const float2 even = mul2(dup(w), add(mul2(rho, sub2(q, usq)), drho));
+  const float2 odd = mul2(mul2(mul2(dup(w), rho), dup(3.0f)), cu);
+  const float2 s_even = mul2(dup(guo * w), add(mul2(mul2(dup(9.0f), cu), dup(cf)), sym_f));
+  const float2 s_odd = dup(guo * w * 3.0f * cf);
+  gi = add(add(mul2(om, sub2(add(even, odd), gi)), gi), add(s_even, s_odd));
+  go = add(add(mul2(om, sub2(sub2(even, odd), go)), go), sub2(s_even, s_odd));
+}
+__device__ __forceinline__ void collide2_forced(float om1, float guo, float fx, float fy,
+                                                float one1, float2 drho, float2 rho, float2 inv,
+                                                float2 g[kQ]) {
+  const float2 om = dup(om1), one = dup(one1);
+  auto add = [&](float2 a, float2 b) { return fma2(a, one, b); };
+  const float2 jx = add2(add2(add2(sub2(g[1], g[3]), sub2(g[5], g[6])), sub2(g[8], g[7])), dup(0.5f * fx));
+  const float2 jy = add2(add2(add2(sub2(g[2], g[4]), sub2(g[5], g[8])), sub2(g[6], g[7])), dup(0.5f * fy));
+  const float2 ux = mul2(jx, inv), uy = mul2(jy, inv);
+  const float2 usq = mul2(dup(1.5f), add(mul2(ux, ux), mul2(uy, uy)));
+  const float2 sym_f = mul2(dup(-3.0f), add(mul2(ux, dup(fx)), mul2(uy, dup(fy))));
+  g[0] = add(add(mul2(om, sub2(mul2(dup(kW0), sub2(drho, mul2(rho, usq))), g[0])), g[0]),
+             mul2(dup(guo * kW0), sym_f));
+  forced_pair2(g[1], g[3], kW1, ux, fx, drho, rho, usq, om, sym_f, guo, one);
+  forced_pair2(g[2], g[4], kW1, uy, fy, drho, rho, usq, om, sym_f, guo, one);
+  forced_pair2(g[5], g[7], kW2, add(ux, uy), fx + fy, drho, rho, usq, om, sym_f, guo, one);
+  forced_pair2(g[6], g[8], kW2, sub2(uy, ux), fy - fx, drho, rho, usq, om, sym_f, guo, one);
+}
+
 __device__ __forceinline__ float get2(const float2 v[kH], int j) {
   return j == 0 ? v[0].x : (j == 1 ? v[0].y : (j == 2 ? v[1].x : v[1].y));
 }
@@ -210,45 +243,37 @@ __device__ __forceinline__ void complete_ends(float dw, float de, int kinds, boo
 }
 
 template <bool FORCED>
-__device__ __forceinline__ void collide_lane(const GridDev* __restrict__ G, float om,
+__device__ __forceinline__ void collide_lane(const GridDev* __restrict__ G, float om, float one,
                                              float2 g[kQ][kH]) {
-  bool scalar = false;  // body force: the scalar code (packed products that feed sums contract)
-  if constexpr (FORCED) scalar = __ldg(&G->fx) != 0.0f || __ldg(&G->fy) != 0.0f;
-  if (!scalar) {
-    float2 drho[kH], rho[kH], inv[kH];
+  bool forced = false;
+  float guo = 0.0f, fx = 0.0f, fy = 0.0f;
+  if constexpr (FORCED) {
+    fx = __ldg(&G->fx);
+    fy = __ldg(&G->fy);
+    guo = __ldg(&G->guo);
+    forced = fx != 0.0f || fy != 0.0f;
+  }
+  float2 drho[kH], rho[kH], inv[kH];
 #pragma unroll
-    for (int h = 0; h < kH; ++h) {
-      float2 c[kQ];
+  for (int h = 0; h < kH; ++h) {
+    float2 c[kQ];
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) c[i] = g[i][h];
-      drho[h] = drho2(c);
-      rho[h] = add2(dup(1.0f), drho[h]);
-    }
-    rcp_lane(rho, inv);
+    for (int i = 0; i < kQ; ++i) c[i] = g[i][h];
+    drho[h] = drho2(c);
+    rho[h] = add2(dup(1.0f), drho[h]);
+  }
+  rcp_lane(rho, inv);
 #pragma unroll
-    for (int h = 0; h < kH; ++h) {
-      float2 c[kQ];
+  for (int h = 0; h < kH; ++h) {
+    float2 c[kQ];
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) c[i] = g[i][h];
+    for (int i = 0; i < kQ; ++i) c[i] = g[i][h];
+    if (!FORCED || !forced)
       collide2(om, drho[h], rho[h], inv[h], c);
+    else
+      collide2_forced(om, guo, fx, fy, one, drho[h], rho[h], inv[h], c);
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) g[i][h] = c[i];
-    }
-  } else {
-    GridDev q;
-    q.omega = om;
-    q.guo = __ldg(&G->guo);
-    q.fx = __ldg(&G->fx);
-    q.fy = __ldg(&G->fy);
-#pragma unroll
-    for (int j = 0; j < kV; ++j) {
-      float c[kQ];
-#pragma unroll
-      for (int i = 0; i < kQ; ++i) c[i] = get2(g[i], j);
-      collide(q, c);
-#pragma unroll
-      for (int i = 0; i < kQ; ++i) set2(g[i], j, c[i]);
-    }
+    for (int i = 0; i < kQ; ++i) g[i][h] = c[i];
   }
 }
 
@@ -287,6 +312,13 @@ __device__ __forceinline__ void pull_row(uint32_t w, uint32_t own, const float2 
   }
 }
 
+// Column of a periodic row: x < nx + kV, without a division (rows shorter than a chunk wrap
+// more than once).
+__device__ __forceinline__ int wrapped(int x, int nx) {
+  while (x >= nx) x -= nx;
+  return x;
+}
+
 // The bits of three consecutive windows of hist.
 constexpr uint32_t kNear = 0x010101u * ((1u << (kV + 2)) - 1u);
 
@@ -294,7 +326,7 @@ template <bool FORCED>
 __global__ void __launch_bounds__(kWarps * 32, kCtas)
     k_sweep(const GridDev* __restrict__ grids, const SweepTask* __restrict__ tasks,
             const uint32_t* __restrict__ mask, const float* __restrict__ src,
-            float* __restrict__ dst, unsigned P) {
+            float* __restrict__ dst, unsigned P, float one) {
   extern __shared__ __align__(128) float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const SweepTask* tkp = tasks + (blockIdx.x * kWarps + warp);
@@ -314,8 +346,8 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
   int p = x, pl, pr;
   bool chunk, west = false;
   unsigned je = kV;
+  const int nx = __ldg(&G->nx);
   {
-    const int nx = __ldg(&G->nx);
     const bool periodic = __ldg(&G->periodic_x) != 0;
     if (periodic) {
       p %= nx;
@@ -353,7 +385,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
     return reinterpret_cast<float*>(reinterpret_cast<char*>(dst + (size_t)i * P) + off);
   };
   const int outs = (x >= tkp->xs && x < tkp->xe) ? (tkp->xe - x < kV ? tkp->xe - x : kV) : 0;
-  uint32_t mw[3] = {0u, 0u, 0u};
+  uint32_t mw[4] = {0u, 0u, 0u, 0u};
   // Copies one row's populations of the classes in `which` (bit 0: 2, 5, 6; bit 1: 0, 1, 3;
   // bit 2: 4, 7, 8) into shared memory; slot: of the two-row classes.
   auto load = [&](uint32_t row, int which, int slot) {
@@ -365,10 +397,9 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
         cpa16(own0 + at * R + (cls_of(i) == 1 ? 0 : slot * 3 * R), from(i, row));
       }
     } else if (active) {
-      const int nx = __ldg(&G->nx);
 #pragma unroll 1
       for (int j = 0; j < kV; ++j) {
-        const uint32_t r = row + 4u * (uint32_t)((p + j) % nx - p);
+        const uint32_t r = row + 4u * (uint32_t)(wrapped(p + j, nx) - p);
 #pragma unroll
         for (int i = 0; i < kQ; ++i) {
           if (!((which >> cls_of(i)) & 1)) continue;
@@ -393,15 +424,11 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
       mw[0] = __ldg(mp + (pl >> 5));
       mw[1] = __ldg(mp + (p >> 5));
       mw[2] = __ldg(mp + (pr >> 5));
-    } else {
-      const int nx = __ldg(&G->nx);
-      uint32_t w = 0;
-#pragma unroll 1
-      for (int b = 0; b < kV + 2; ++b) {
-        const int q = (p + nx - 1 + b) % nx;
-        w |= ((__ldg(mp + (q >> 5)) >> (q & 31)) & 1u) << b;
-      }
-      mw[0] = w;
+    } else {  // the row wraps inside the chunk or it is unaligned: words only, no dependent loads
+      mw[0] = __ldg(mp + (pl >> 5));
+      mw[1] = __ldg(mp + (p >> 5));
+      mw[2] = __ldg(mp + (min(p + kV, nx - 1) >> 5));
+      mw[3] = __ldg(mp);
     }
   };
   auto next_row = [&]() {  // advance the input row by one
@@ -416,7 +443,21 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
   // solid bits of the row whose mask words were loaded last (those beyond an open end are
   // bits of other cells: they only reach populations that the completion replaces)
   auto window = [&]() -> uint32_t {
-    if (!chunk) return mw[0];
+    if (!chunk) {
+      uint32_t v = mw[1] >> (p & 31);  // cells p ... of the row
+      if ((p & 31) > 32 - (kV + 1)) v |= mw[2] << (32 - (p & 31));
+      const int in = nx - p;  // ... those before the wrap, then cells 0 ...
+      if (in < kV + 1) {
+        uint32_t w = mw[3];
+        if (nx < kV) {  // rows that wrap more than once
+          w &= (1u << nx) - 1u;
+          w |= w << nx;
+          w |= w << (2 * nx);
+        }
+        v = (v & ((1u << in) - 1u)) | (w << in);
+      }
+      return ((mw[0] >> (pl & 31)) & 1u) | ((v & ((1u << (kV + 1)) - 1u)) << 1);
+    }
     return ((mw[0] >> (pl & 31)) & 1u) | (((mw[1] >> (p & 31)) & kOwn) << 1) |
            (((mw[2] >> (pr & 31)) & 1u) << (kV + 1));
   };
@@ -519,7 +560,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
         cpa_commit();
       }
       if (at_end) complete_ends(dw, de, kinds, west, je, g);
-      collide_lane<FORCED>(G, om, g);
+      collide_lane<FORCED>(G, om, one, g);
       if (t == kT) {  // the pass's result: solid cells store 0
         if (outs) {
           const uint32_t own = w >> 9;
@@ -611,7 +652,7 @@ void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks) {
   // Rows a task advances: the cut whose waves of CTAs take the fewest row steps.  A task of l
   // rows costs l + 3 row iterations of level 2 (l + 2 of level 1) and a start of about two
   // more, so many small cuts lose to one wave of large ones: 64 grids of 512 x 256 at 36 rows
-  // (one wave of 448 CTAs) 57.8 us a step, at 30 rows (1.3 waves) 72.4, at 64 rows 96.2.
+  // (one wave of 448 CTAs) 58 us a step, at 30 rows (1.3 waves) 72, at 64 rows 96.
   int max_ny = 0;
   std::vector<Strips> strips;
   for (const GridDev& d : gd) {
@@ -687,6 +728,23 @@ void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks) {
   while (tasks->size() % kWarps) tasks->push_back(SweepTask{});
 }
 
+// Periodic rows of a length that is no multiple of 4 wrap inside a chunk: every row of such a
+// warp copies its wrapped cells one by one, so its tasks end last, and rows up to two warps long
+// have no other warps to hide it; with a body force, whose collision is longer, longer rows lose
+// as well.  Measured against single steps: 0.89 to 1.11 of the speed on 1 .. 50 grids of 33 ..
+// 230 columns; from 256 columns on 1.0 to 1.3 without a force, 0.78 to 1.07 with one.  So a
+// batch most of whose cells lie in such rows steps singly.
+bool sweep_pays(const std::vector<GridDev>& gd) {
+  long long narrow = 0, all = 0;
+  for (const GridDev& d : gd) {
+    const long long cells = (long long)d.nx * d.ny;
+    all += cells;
+    const bool forced = d.fx != 0.0f || d.fy != 0.0f;
+    if (d.periodic_x && d.nx % kV != 0 && (d.nx < 256 || forced)) narrow += cells;
+  }
+  return 2 * narrow <= all;
+}
+
 int sweep_init() {
   cudaError_t e = cudaFuncSetAttribute(k_sweep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kSmem);
@@ -712,7 +770,7 @@ int sweep_launch(Handle* h, const float* src, float* dst, cudaStream_t s) {
   auto kernel = forced ? k_sweep<true> : k_sweep<false>;
   LBM_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, (const GridDev*)h->gd_d,
                                     (const SweepTask*)h->sweep_d, (const uint32_t*)h->mask, src,
-                                    dst, (unsigned)h->gd[0].plane));
+                                    dst, (unsigned)h->gd[0].plane, 1.0f));
   return LBM_OK;
 }
 
