@@ -463,70 +463,113 @@ __global__ void __launch_bounds__(kLiftThreads, lift_ctas_per_sm(kCin, kC))
   if (warp == 0) tmem_dealloc(tmem, 2 * kAccCols);
 }
 
-// Projection Q from the channel-blocked field, any decoder shape (the common shape
-// runs in k_decoder_tc); one thread per pixel of the output grid H0 x W0 (the padded
-// grid is cropped), decoder weights staged in shared memory.
-template <int kC>
+// Projection Q from the channel-blocked field for the decoders k_decoder_tc does not take (several
+// hidden layers, other widths); FP32 throughout.  A thread owns kNP pixels of the output grid (the
+// padded grid is cropped): its hidden units stay in registers, packed over pairs of inputs, and
+// every 16-byte broadcast load of weights from shared memory feeds 2 kNP packed multiply-adds, which
+// bound it.  Widths below kS are padded with zero weights.  (Hidden units in indexed arrays, as
+// they were, live in local memory: three layers of 32 on 256 x 512 pixels took 110 us.)
+template <int kF2, int kS, int kNP>
+__device__ __forceinline__ void dec_layer(const float* w, const float* bias, int act,
+                                          const float2 (*in)[kF2], float2 (*out)[kS / 2]) {
+#pragma unroll
+  for (int j = 0; j < kS; j += 2) {
+    float2 acc[kNP][2];
+#pragma unroll
+    for (int q = 0; q < kNP; ++q) acc[q][0] = acc[q][1] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int c = 0; c < kF2; c += 2) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float4 v = *reinterpret_cast<const float4*>(w + (j + u) * 2 * kF2 + 2 * c);
+#pragma unroll
+        for (int q = 0; q < kNP; ++q) {
+          acc[q][u] = __ffma2_rn(make_float2(v.x, v.y), in[q][c], acc[q][u]);
+          acc[q][u] = __ffma2_rn(make_float2(v.z, v.w), in[q][c + 1], acc[q][u]);
+        }
+      }
+    }
+    const float2 bj = *reinterpret_cast<const float2*>(bias + j);
+#pragma unroll
+    for (int q = 0; q < kNP; ++q) {
+      const float2 v = make_float2(acc[q][0].x + acc[q][0].y + bj.x, acc[q][1].x + acc[q][1].y + bj.y);
+      out[q][j / 2] = act == FNO_ACT_GELU ? gelu_poly2(v) : make_float2(act_tc(v.x, act), act_tc(v.y, act));
+    }
+  }
+}
+template <int kC, int kS, int kNP>
 __global__ void __launch_bounds__(128)
-    k_decoder_blk(const __nv_bfloat16* __restrict__ theta, float* __restrict__ out,
-                  const float* __restrict__ params, const unsigned* __restrict__ offs,
-                  int nlayers, int B, TcGrid gd, int S, int cout, int act) {
+    k_decoder_deep(const __nv_bfloat16* __restrict__ theta, float* __restrict__ out,
+                   const float* __restrict__ params, const unsigned* __restrict__ offs,
+                   int nlayers, int B, TcGrid gd, int S, int cout, int act) {
+  extern __shared__ __align__(16) float dec_s[];
   pdl_trigger();
-  pdl_wait();
-  const int H = gd.H0, W = gd.W0;
-  extern __shared__ float dec_s[];
-  // layout: for each layer l: w [S][fan] then b [S]; then out.w [cout][fan], out.b [cout]
-  int at = 0, fan = kC;
-  for (int l = 0; l <= nlayers; ++l) {
-    const int rows = l < nlayers ? S : cout;
+  // layout: w of layer 0 [kS][kC], of the others [kS][kS], out.w [cout][kS]; their biases [kS]
+  float* const bias_s = dec_s + kS * kC + (nlayers - 1) * kS * kS + cout * kS;
+  for (int l = 0, at = 0, fan = kC; l <= nlayers; ++l) {
+    const int rows = l < nlayers ? kS : cout, have = l < nlayers ? S : cout;
+    const int src_fan = l == 0 ? kC : S;
     const float* w = params + offs[2 * l];
     const float* bb = params + offs[2 * l + 1];
-    for (int t = threadIdx.x; t < rows * fan; t += blockDim.x) dec_s[at + t] = w[t];
-    for (int t = threadIdx.x; t < rows; t += blockDim.x) dec_s[at + rows * fan + t] = bb[t];
-    at += rows * fan + rows;
-    fan = S;
+    for (int t = threadIdx.x; t < rows * fan; t += blockDim.x) {
+      const int j = t / fan, c = t - j * fan;
+      dec_s[at + t] = j < have && c < src_fan ? w[j * src_fan + c] : 0.0f;
+    }
+    for (int t = threadIdx.x; t < rows; t += blockDim.x) bias_s[l * kS + t] = t < have ? bb[t] : 0.0f;
+    at += rows * fan;
+    fan = kS;
   }
+  pdl_wait();
   __syncthreads();
+  const int H = gd.H0, W = gd.W0;
   const size_t pix = (size_t)B * H * W;
-  const size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (p >= pix) return;
-  const int x = (int)(p % W);
-  const int y = (int)((p / W) % H);
-  const int b = (int)(p / ((size_t)W * H));
-  const size_t row = (size_t)b * gd.Hs + y;  // storage row
-  float a[kC];
+  const size_t p0 = blockIdx.x * (size_t)(128 * kNP) + threadIdx.x;
+  float2 h[kNP][kS / 2], t[kNP][kS / 2];
+  size_t at_out[kNP];
+  float2 a[kNP][kC / 2];
 #pragma unroll
-  for (int g = 0; g < kC / 8; ++g) {
-    const uint4 v = *reinterpret_cast<const uint4*>(theta + ((row * (kC / 8) + g) * gd.Ws + x) * 8);
-    const __nv_bfloat16* hv = reinterpret_cast<const __nv_bfloat16*>(&v);
+  for (int q = 0; q < kNP; ++q) {
+    const size_t p = min(p0 + (size_t)q * 128, pix - 1);
+    const int x = (int)(p % W);
+    const int y = (int)((p / W) % H);
+    const int b = (int)(p / ((size_t)W * H));
+    at_out[q] = ((size_t)b * cout * H + y) * W + x;
+    const size_t row = (size_t)b * gd.Hs + y;  // storage row
 #pragma unroll
-    for (int q = 0; q < 8; ++q) a[g * 8 + q] = __bfloat162float(hv[q]);
+    for (int g = 0; g < kC / 8; ++g) {
+      const uint4 v = *reinterpret_cast<const uint4*>(theta + ((row * (kC / 8) + g) * gd.Ws + x) * 8);
+      const __nv_bfloat162* hv = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[q][g * 4 + u] = __bfloat1622float2(hv[u]);
+    }
   }
-  {
-    float h[64], t[64];
+  dec_layer<kC / 2, kS, kNP>(dec_s, bias_s, act, a, h);
+  const float* w = dec_s + kS * kC;
+#pragma unroll 1
+  for (int l = 1; l < nlayers; ++l, w += kS * kS) {
+    dec_layer<kS / 2, kS, kNP>(w, bias_s + l * kS, act, h, t);
 #pragma unroll
-    for (int c = 0; c < kC; ++c) h[c] = a[c];
-    at = 0;
-    fan = kC;
-    for (int l = 0; l < nlayers; ++l) {
-      const float* w = dec_s + at;
-      const float* bb = w + S * fan;
-      for (int j = 0; j < S; ++j) {
-        float v = bb[j];
-        for (int c = 0; c < fan; ++c) v = fmaf(w[j * fan + c], h[c], v);
-        t[j] = act_tc(v, act);
+    for (int q = 0; q < kNP; ++q)
+#pragma unroll
+      for (int c = 0; c < kS / 2; ++c) h[q][c] = t[q][c];
+  }
+#pragma unroll 1
+  for (int o = 0; o < cout; ++o) {
+    float2 acc[kNP];
+#pragma unroll
+    for (int q = 0; q < kNP; ++q) acc[q] = make_float2(bias_s[nlayers * kS + o], 0.0f);
+#pragma unroll
+    for (int c = 0; c < kS / 2; c += 2) {
+      const float4 v = *reinterpret_cast<const float4*>(w + o * kS + 2 * c);
+#pragma unroll
+      for (int q = 0; q < kNP; ++q) {
+        acc[q] = __ffma2_rn(make_float2(v.x, v.y), h[q][c], acc[q]);
+        acc[q] = __ffma2_rn(make_float2(v.z, v.w), h[q][c + 1], acc[q]);
       }
-      for (int j = 0; j < S; ++j) h[j] = t[j];
-      at += S * fan + S;
-      fan = S;
     }
-    const float* w = dec_s + at;
-    const float* bb = w + cout * fan;
-    for (int q = 0; q < cout; ++q) {
-      float v = bb[q];
-      for (int c = 0; c < fan; ++c) v = fmaf(w[q * fan + c], h[c], v);
-      out[(((size_t)b * cout + q) * H + y) * W + x] = v;
-    }
+#pragma unroll
+    for (int q = 0; q < kNP; ++q)
+      if (p0 + (size_t)q * 128 < pix) out[at_out[q] + (size_t)o * H * W] = acc[q].x + acc[q].y;
   }
 }
 
@@ -1734,12 +1777,19 @@ static int fno_forward_tc_impl(const fno_config& c, const FnoTcParams& P, const 
       LBM_TRY(launch_pdl((k_decoder_tc<kC, 64, kAct>), dim3(ctas), dim3(kDecThreads), smem_tc, s,
                          th[cur], out, P.params, P.dec_offs, B, gd, c.c_out, status));
   } else {
+    const int S = c.dec_size <= 32 ? 32 : 64, np = S == 32 ? 2 : 1;
     const size_t dec_smem =
-        ((size_t)c.dec_layers * (c.dec_size * 64 + c.dec_size) + c.c_out * 64 + c.c_out) *
-        sizeof(float);
-    LBM_TRY(launch_pdl((k_decoder_blk<kC>), dim3((unsigned)((pix + 127) / 128)), dim3(128), dec_smem, s, 
-        th[cur], out, P.params, P.dec_offs, c.dec_layers, B, gd, c.dec_size, c.c_out,
-        c.activation));
+        ((size_t)S * kC + (size_t)(c.dec_layers - 1) * S * S + (size_t)c.c_out * S +
+         (size_t)(c.dec_layers + 1) * S) * sizeof(float);
+    const dim3 blocks((unsigned)((pix + 128 * np - 1) / (128 * np)));
+    if (S == 32)
+      LBM_TRY(launch_pdl((k_decoder_deep<kC, 32, 2>), blocks, dim3(128), dec_smem, s, th[cur], out,
+                         P.params, P.dec_offs, c.dec_layers, B, gd, c.dec_size, c.c_out,
+                         c.activation));
+    else
+      LBM_TRY(launch_pdl((k_decoder_deep<kC, 64, 1>), blocks, dim3(128), dec_smem, s, th[cur], out,
+                         P.params, P.dec_offs, c.dec_layers, B, gd, c.dec_size, c.c_out,
+                         c.activation));
   }
   return LBM_OK;
 }
@@ -1781,7 +1831,10 @@ static int tc_set_smem_attrs() {
   if constexpr (kC <= 32)
     LBM_CHECK_CUDA(cudaFuncSetAttribute(k_mix4<kC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         kTcSmemMax));
-  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_decoder_blk<kC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemMax));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_decoder_deep<kC, 32, 2>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemMax));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_decoder_deep<kC, 64, 1>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemMax));
   LBM_TRY((tc_set_smem_attrs_act<kC, FNO_ACT_GELU>()));
   return tc_set_smem_attrs_act<kC, FNO_ACT_RELU>();
 }
