@@ -469,18 +469,22 @@ __global__ void __launch_bounds__(kLiftThreads, lift_ctas_per_sm(kCin, kC))
 // every 16-byte broadcast load of weights from shared memory feeds 2 kNP packed multiply-adds, which
 // bound it.  Widths below kS are padded with zero weights.  (Hidden units in indexed arrays, as
 // they were, live in local memory: three layers of 32 on 256 x 512 pixels took 110 us.)
-template <int kF2, int kS, int kNP>
-__device__ __forceinline__ void dec_layer(const float* w, const float* bias, int act,
-                                          const float2 (*in)[kF2], float2 (*out)[kS / 2]) {
+// The layer loop stays rolled: four outputs at a time go to the thread's own column of shared
+// memory (conflict-free) and are read back as the next layer's inputs.
+template <int kF2, int kNP>
+__device__ __forceinline__ void dec_layer(const float* w, const float* bias, int S, int act,
+                                          const float2 (*in)[kF2], float* col) {
+#pragma unroll 1
+  for (int j = 0; j < S; j += 4) {
+    float2 acc[kNP][4];
 #pragma unroll
-  for (int j = 0; j < kS; j += 2) {
-    float2 acc[kNP][2];
+    for (int q = 0; q < kNP; ++q)
 #pragma unroll
-    for (int q = 0; q < kNP; ++q) acc[q][0] = acc[q][1] = make_float2(0.0f, 0.0f);
+      for (int u = 0; u < 4; ++u) acc[q][u] = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int c = 0; c < kF2; c += 2) {
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < 4; ++u) {
         const float4 v = *reinterpret_cast<const float4*>(w + (j + u) * 2 * kF2 + 2 * c);
 #pragma unroll
         for (int q = 0; q < kNP; ++q) {
@@ -489,11 +493,23 @@ __device__ __forceinline__ void dec_layer(const float* w, const float* bias, int
         }
       }
     }
-    const float2 bj = *reinterpret_cast<const float2*>(bias + j);
+    const float4 bj = *reinterpret_cast<const float4*>(bias + j);
 #pragma unroll
     for (int q = 0; q < kNP; ++q) {
-      const float2 v = make_float2(acc[q][0].x + acc[q][0].y + bj.x, acc[q][1].x + acc[q][1].y + bj.y);
-      out[q][j / 2] = act == FNO_ACT_GELU ? gelu_poly2(v) : make_float2(act_tc(v.x, act), act_tc(v.y, act));
+      float2 v0 = make_float2(acc[q][0].x + acc[q][0].y + bj.x, acc[q][1].x + acc[q][1].y + bj.y);
+      float2 v1 = make_float2(acc[q][2].x + acc[q][2].y + bj.z, acc[q][3].x + acc[q][3].y + bj.w);
+      if (act == FNO_ACT_GELU) {
+        v0 = gelu_poly2(v0);
+        v1 = gelu_poly2(v1);
+      } else {
+        v0 = make_float2(act_tc(v0.x, act), act_tc(v0.y, act));
+        v1 = make_float2(act_tc(v1.x, act), act_tc(v1.y, act));
+      }
+      float* o = col + (q * S + j) * 128;
+      o[0] = v0.x;
+      o[128] = v0.y;
+      o[256] = v1.x;
+      o[384] = v1.y;
     }
   }
 }
@@ -524,7 +540,7 @@ __global__ void __launch_bounds__(128)
   const int H = gd.H0, W = gd.W0;
   const size_t pix = (size_t)B * H * W;
   const size_t p0 = blockIdx.x * (size_t)(128 * kNP) + threadIdx.x;
-  float2 h[kNP][kS / 2], t[kNP][kS / 2];
+  float2 h[kNP][kS / 2];
   size_t at_out[kNP];
   float2 a[kNP][kC / 2];
 #pragma unroll
@@ -543,15 +559,21 @@ __global__ void __launch_bounds__(128)
       for (int u = 0; u < 4; ++u) a[q][g * 4 + u] = __bfloat1622float2(hv[u]);
     }
   }
-  dec_layer<kC / 2, kS, kNP>(dec_s, bias_s, act, a, h);
-  const float* w = dec_s + kS * kC;
-#pragma unroll 1
-  for (int l = 1; l < nlayers; ++l, w += kS * kS) {
-    dec_layer<kS / 2, kS, kNP>(w, bias_s + l * kS, act, h, t);
+  float* const col = bias_s + (nlayers + 1) * kS + threadIdx.x;  // [kNP][kS][128]
+  auto reload = [&]() {
 #pragma unroll
     for (int q = 0; q < kNP; ++q)
 #pragma unroll
-      for (int c = 0; c < kS / 2; ++c) h[q][c] = t[q][c];
+      for (int c = 0; c < kS / 2; ++c)
+        h[q][c] = make_float2(col[(q * kS + 2 * c) * 128], col[(q * kS + 2 * c + 1) * 128]);
+  };
+  dec_layer<kC / 2, kNP>(dec_s, bias_s, kS, act, a, col);
+  reload();
+  const float* w = dec_s + kS * kC;
+#pragma unroll 1
+  for (int l = 1; l < nlayers; ++l, w += kS * kS) {
+    dec_layer<kS / 2, kNP>(w, bias_s + l * kS, kS, act, h, col);
+    reload();
   }
 #pragma unroll 1
   for (int o = 0; o < cout; ++o) {
@@ -1780,7 +1802,7 @@ static int fno_forward_tc_impl(const fno_config& c, const FnoTcParams& P, const 
     const int S = c.dec_size <= 32 ? 32 : 64, np = S == 32 ? 2 : 1;
     const size_t dec_smem =
         ((size_t)S * kC + (size_t)(c.dec_layers - 1) * S * S + (size_t)c.c_out * S +
-         (size_t)(c.dec_layers + 1) * S) * sizeof(float);
+         (size_t)(c.dec_layers + 1) * S + (size_t)np * S * 128) * sizeof(float);
     const dim3 blocks((unsigned)((pix + 128 * np - 1) / (128 * np)));
     if (S == 32)
       LBM_TRY(launch_pdl((k_decoder_deep<kC, 32, 2>), blocks, dim3(128), dec_smem, s, th[cur], out,
