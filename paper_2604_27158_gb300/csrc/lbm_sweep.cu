@@ -24,7 +24,7 @@
 // the same order; the file is compiled without multiply-add contraction.  States are bitwise
 // those of single steps.
 //
-// What bounds it (64 grids of 512 x 256): 58 us a step.  The pass moves 5.2 TB/s; issue
+// What bounds it (64 grids of 512 x 256): 57 us a step.  The pass moves 5.3 TB/s; issue
 // slots are 46% busy with the eleven warps a multiprocessor that the shared memory of the
 // kept rows allows, and their fixed-latency chains are what is left.  Measured and not kept:
 // two cells a lane and 24 warps (89 us: the per-lane work is not halved), the kept rows in
@@ -107,6 +107,11 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 // a * b as the fused a * b - 0, which cannot be contracted with an addition that follows
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return fma2(a, b, dup(-0.0f)); }
+// A constant times a pair as two scalar products: they take the constant as an immediate, which
+// packed instructions do not (58.3 -> 57.0 us a step on 64 grids of 512 x 256).
+__device__ __forceinline__ float2 mulc(float c, float2 a) {
+  return make_float2(__fmul_rn(c, a.x), __fmul_rn(c, a.y));
+}
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, dup(-1.0f), a); }
 
 // Correctly rounded reciprocals of a lane's values, all in [0.5, 2): the approximate
@@ -152,14 +157,14 @@ __device__ __forceinline__ void collide2(float om1, float2 drho, float2 rho, flo
   const float2 jx = add2(add2(sub2(g[1], g[3]), sub2(g[5], g[6])), sub2(g[8], g[7]));
   const float2 jy = add2(add2(sub2(g[2], g[4]), sub2(g[5], g[8])), sub2(g[6], g[7]));
   const float2 ux = mul2(jx, inv), uy = mul2(jy, inv);
-  const float2 rusq = mul2(mul2(rho, dup(1.5f)), fma2(ux, ux, mul2(uy, uy)));
+  const float2 rusq = mul2(mulc(1.5f, rho), fma2(ux, ux, mul2(uy, uy)));
   const float2 d = sub2(drho, rusq);
-  const float2 e1 = mul2(dup(kW1), d), e2 = mul2(dup(kW2), d);
-  const float2 r1 = mul2(dup(kW1), rho), r2 = mul2(dup(kW2), rho);
-  const float2 a1 = mul2(dup(3.0f), r1), a2 = mul2(dup(3.0f), r2);
-  const float2 n1 = mul2(dup(-1.0f), a1), n2 = mul2(dup(-1.0f), a2);
-  const float2 b1 = mul2(dup(4.5f), r1), b2 = mul2(dup(4.5f), r2);
-  g[0] = fma2(om, fma2(dup(kW0), d, mul2(dup(-1.0f), g[0])), g[0]);
+  const float2 e1 = mulc(kW1, d), e2 = mulc(kW2, d);
+  const float2 r1 = mulc(kW1, rho), r2 = mulc(kW2, rho);
+  const float2 a1 = mulc(3.0f, r1), a2 = mulc(3.0f, r2);
+  const float2 n1 = mulc(-1.0f, a1), n2 = mulc(-1.0f, a2);
+  const float2 b1 = mulc(4.5f, r1), b2 = mulc(4.5f, r2);
+  g[0] = fma2(om, fma2(dup(kW0), d, mulc(-1.0f, g[0])), g[0]);
   relax_pair2(g[1], g[3], a1, n1, b1, ux, e1, om);
   relax_pair2(g[2], g[4], a1, n1, b1, uy, e1, om);
   relax_pair2(g[5], g[7], a2, n2, b2, add2(ux, uy), e2, om);
@@ -260,7 +265,7 @@ __device__ __forceinline__ void collide_lane(const GridDev* __restrict__ G, floa
 #pragma unroll
     for (int i = 0; i < kQ; ++i) c[i] = g[i][h];
     drho[h] = drho2(c);
-    rho[h] = add2(dup(1.0f), drho[h]);
+    rho[h] = make_float2(__fadd_rn(1.0f, drho[h].x), __fadd_rn(1.0f, drho[h].y));
   }
   rcp_lane(rho, inv);
 #pragma unroll
