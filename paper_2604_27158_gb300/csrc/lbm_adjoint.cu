@@ -150,6 +150,29 @@ __global__ void __launch_bounds__(kBlock) k_adj_macro(const GridDev* __restrict_
   store9(Gc, mu, x, y, m);
 }
 
+// Solid bits of cells x - 1, x, x + 1 of mask row mr (bits 0, 1, 2), wrapped for periodic rows, 0
+// beyond an open end.  The cells of a warp share their word, so these are broadcast loads.
+__device__ __forceinline__ uint32_t cell_window(const uint32_t* __restrict__ mr, const GridDev& G,
+                                                int x) {
+  const int wi = x >> 5;
+  uint64_t v = (uint64_t)__ldg(mr + wi) << 1;
+  if (wi > 0) v |= __ldg(mr + wi - 1) >> 31;
+  if (wi + 1 < G.wpr) v |= (uint64_t)(__ldg(mr + wi + 1) & 1u) << 33;
+  uint32_t win = (uint32_t)(v >> (x & 31)) & 7u;
+  if (x == 0) {
+    win &= 6u;
+    if (G.periodic_x) win |= (uint32_t)mask_bit(mr, 0, G.nx - 1, 0);
+  }
+  if (x == G.nx - 1) {
+    win &= 3u;
+    if (G.periodic_x) win |= (uint32_t)mask_bit(mr, 0, 0, 0) << 2;
+  }
+  return win;
+}
+
+// One cell a thread, both gathers from three 3-bit windows of the mask and one selected address a
+// population, all eighteen loads in flight at once (with a mask word and an address of its own for
+// every neighbour, as pull_cell does it: 74 us on 2.1 M cells, now 71; HBM needs 33).
 __global__ void __launch_bounds__(kBlock) k_adj_step(const GridDev* __restrict__ grids,
                                                      int ngrids, const uint32_t* __restrict__ mask,
                                                      const float* __restrict__ state_prev,
@@ -158,47 +181,49 @@ __global__ void __launch_bounds__(kBlock) k_adj_step(const GridDev* __restrict__
   int gidx, x, y;
   if (!cell_of_thread(grids, ngrids, gidx, x, y)) return;
   const GridDev Gc = canonical(grids[gidx]);
+  const int ym = (y == 0) ? Gc.ny - 1 : y - 1, yp = (y == Gc.ny - 1) ? 0 : y + 1;
+  const uint32_t* m = mask + Gc.mask_off;
+  const uint32_t win[3] = {cell_window(m + (size_t)ym * Gc.wpr, Gc, x),
+                           cell_window(m + (size_t)y * Gc.wpr, Gc, x),
+                           cell_window(m + (size_t)yp * Gc.wpr, Gc, x)};
   float f[kQ], l[kQ];
-  if (!pull_cell(Gc, mask, state_prev, x, y, f)) {
+  if (win[1] & 2u) {
 #pragma unroll
     for (int i = 0; i < kQ; ++i) l[i] = 0.0f;
     store9(Gc, mu_out, x, y, l);
     return;
   }
-  // G^T: slot (j, x) of the stored state was read by cell x + c_j as its population j
-  // when that cell is a fluid cell of the domain, by this cell's population opp(j)
-  // (bounce-back) when it is solid, and by nobody when it lies beyond an open end.
-  const uint32_t* m = mask + Gc.mask_off;
-  const float* b = mu_in + Gc.f_off;
-  const long long P = Gc.plane;
-  const long long here = (long long)y * Gc.pitch + x;
-  const int yp = (y == Gc.ny - 1) ? 0 : y + 1;
-  const int ym = (y == 0) ? Gc.ny - 1 : y - 1;
-  l[0] = b[here];
+  const bool west_end = x == 0, east_end = x == Gc.nx - 1;
+  const int xm = west_end ? Gc.nx - 1 : x - 1, xp = east_end ? 0 : x + 1;
+  const long long row[3] = {(long long)ym * Gc.pitch, (long long)y * Gc.pitch,
+                            (long long)yp * Gc.pitch};
+  const float* bs = state_prev + Gc.f_off;
+  const float* bm = mu_in + Gc.f_off;
+  // population i of f comes from x - c_i; slot (j, x) of the stored state was read by cell x + c_j
+  // when that is a fluid cell of the domain, by this cell's population opp(j) (bounce-back) when
+  // it is solid, and by nobody when it lies beyond an open end
 #pragma unroll
-  for (int j = 1; j < kQ; ++j) {
-    int tx = x + cx_of(j);
-    const int ty = cy_of(j) == 0 ? y : (cy_of(j) > 0 ? yp : ym);
-    if (tx < 0 || tx >= Gc.nx) {
-      if (!Gc.periodic_x) {
-        l[j] = 0.0f;
-        continue;
-      }
-      tx = tx < 0 ? Gc.nx - 1 : 0;
-    }
-    if (mask_bit(m, Gc.wpr, tx, ty))
-      l[j] = b[(long long)opp_of(j) * P + here];
-    else
-      l[j] = b[(long long)j * P + (long long)ty * Gc.pitch + tx];
+  for (int i = 0; i < kQ; ++i) {
+    const int dx = cx_of(i), dy = cy_of(i);
+    const bool from_out = !Gc.periodic_x && (dx > 0 ? west_end : (dx < 0 && east_end));
+    const bool to_out = !Gc.periodic_x && (dx > 0 ? east_end : (dx < 0 && west_end));
+    const bool from_solid = i > 0 && ((win[1 - dy] >> (1 - dx)) & 1u);
+    const bool to_solid = i > 0 && ((win[1 + dy] >> (1 + dx)) & 1u);
+    const long long from = row[1 - dy] + (dx > 0 ? xm : (dx < 0 ? xp : x));
+    const long long to = row[1 + dy] + (dx > 0 ? xp : (dx < 0 ? xm : x));
+    const long long own = opp_of(i) * Gc.plane + row[1] + x;
+    f[i] = from_out ? 0.0f : __ldg(bs + (from_solid ? own : i * Gc.plane + from));
+    l[i] = to_out ? 0.0f : __ldg(bm + (to_solid ? own : i * Gc.plane + to));
   }
+  complete_cell(Gc, x, f);
   collision_transpose(Gc, f, l);
-  zou_he_transpose(Gc, !Gc.periodic_x && x == 0, !Gc.periodic_x && x == Gc.nx - 1, l);
+  zou_he_transpose(Gc, !Gc.periodic_x && west_end, !Gc.periodic_x && east_end, l);
   store9(Gc, mu_out, x, y, l);
 }
 
 // k_adj_macro with a chunk of four cells a lane, for batches whose canonical and dense rows are
-// 16-byte aligned (2.1 M cells: 64 -> 38 us).  The adjoint step in this form was slower (86 us
-// against 74: both gathers of four cells leave too few warps), so it stays one cell a thread.
+// 16-byte aligned (2.1 M cells: 64 -> 38 us).  The adjoint step in this form took 86 us: both
+// gathers of four cells leave too few warps, so it stays one cell a thread.
 __device__ __forceinline__ void store9_chunk(const GridDev& Gc, float* buf, const ChunkAt& at,
                                              const float v[kQ][4]) {
   float* o = buf + Gc.f_off + (size_t)at.y * Gc.pitch + at.x;
