@@ -172,7 +172,8 @@ __device__ __forceinline__ uint32_t cell_window(const uint32_t* __restrict__ mr,
 
 // One cell a thread, both gathers from three 3-bit windows of the mask and one selected address a
 // population, all eighteen loads in flight at once (with a mask word and an address of its own for
-// every neighbour, as pull_cell does it: 74 us on 2.1 M cells, now 71; HBM needs 33).
+// every neighbour, as pull_cell does it: 74 us on 2.1 M cells, now 62; HBM needs 33, and the 750
+// instructions a cell keep the issue slots 68% busy).
 __global__ void __launch_bounds__(kBlock) k_adj_step(const GridDev* __restrict__ grids,
                                                      int ngrids, const uint32_t* __restrict__ mask,
                                                      const float* __restrict__ state_prev,
@@ -194,9 +195,12 @@ __global__ void __launch_bounds__(kBlock) k_adj_step(const GridDev* __restrict__
     return;
   }
   const bool west_end = x == 0, east_end = x == Gc.nx - 1;
-  const int xm = west_end ? Gc.nx - 1 : x - 1, xp = east_end ? 0 : x + 1;
-  const long long row[3] = {(long long)ym * Gc.pitch, (long long)y * Gc.pitch,
-                            (long long)yp * Gc.pitch};
+  const bool open_w = !Gc.periodic_x && west_end, open_e = !Gc.periodic_x && east_end;
+  // 32-bit indexes from the grid's first value (a batch holds fewer than 2^31)
+  const unsigned xm = west_end ? Gc.nx - 1 : x - 1, xp = east_end ? 0 : x + 1;
+  const unsigned P = (unsigned)Gc.plane, pitch = (unsigned)Gc.pitch;
+  const unsigned row[3] = {(unsigned)ym * pitch, (unsigned)y * pitch, (unsigned)yp * pitch};
+  const unsigned here = row[1] + (unsigned)x;
   const float* bs = state_prev + Gc.f_off;
   const float* bm = mu_in + Gc.f_off;
   // population i of f comes from x - c_i; slot (j, x) of the stored state was read by cell x + c_j
@@ -205,20 +209,22 @@ __global__ void __launch_bounds__(kBlock) k_adj_step(const GridDev* __restrict__
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
     const int dx = cx_of(i), dy = cy_of(i);
-    const bool from_out = !Gc.periodic_x && (dx > 0 ? west_end : (dx < 0 && east_end));
-    const bool to_out = !Gc.periodic_x && (dx > 0 ? east_end : (dx < 0 && west_end));
+    const bool from_out = dx > 0 ? open_w : (dx < 0 && open_e);
+    const bool to_out = dx > 0 ? open_e : (dx < 0 && open_w);
     const bool from_solid = i > 0 && ((win[1 - dy] >> (1 - dx)) & 1u);
     const bool to_solid = i > 0 && ((win[1 + dy] >> (1 + dx)) & 1u);
-    const long long from = row[1 - dy] + (dx > 0 ? xm : (dx < 0 ? xp : x));
-    const long long to = row[1 + dy] + (dx > 0 ? xp : (dx < 0 ? xm : x));
-    const long long own = opp_of(i) * Gc.plane + row[1] + x;
-    f[i] = from_out ? 0.0f : __ldg(bs + (from_solid ? own : i * Gc.plane + from));
-    l[i] = to_out ? 0.0f : __ldg(bm + (to_solid ? own : i * Gc.plane + to));
+    const unsigned from = i * P + row[1 - dy] + (dx > 0 ? xm : (dx < 0 ? xp : (unsigned)x));
+    const unsigned to = i * P + row[1 + dy] + (dx > 0 ? xp : (dx < 0 ? xm : (unsigned)x));
+    const unsigned own = opp_of(i) * P + here;
+    f[i] = from_out ? 0.0f : __ldg(bs + (from_solid ? own : from));
+    l[i] = to_out ? 0.0f : __ldg(bm + (to_solid ? own : to));
   }
   complete_cell(Gc, x, f);
   collision_transpose(Gc, f, l);
-  zou_he_transpose(Gc, !Gc.periodic_x && west_end, !Gc.periodic_x && east_end, l);
-  store9(Gc, mu_out, x, y, l);
+  zou_he_transpose(Gc, open_w, open_e, l);
+  float* o = mu_out + Gc.f_off;
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) o[i * P + here] = l[i];
 }
 
 // k_adj_macro with a chunk of four cells a lane, for batches whose canonical and dense rows are
