@@ -171,8 +171,9 @@ TrPlan tr_plan(const fno_config& c, int B, int H, int W) {
 // erf form took as many issue slots as the 64-channel layer it follows.  NaN propagates.
 __device__ __forceinline__ void tr_gelu2(float2 v, float2* g, float2* d) {
   constexpr float c[GELU_T_DEG + 1] = GELU_T_COEFFS;
-  // beyond 64 the tail is 0; the clamp keeps a Q defined for infinities
-  const float2 a = make_float2(fminf(fabsf(v.x), 64.0f), fminf(fabsf(v.y), 64.0f));
+  // |v|; positive values are clamped to 64, where the tail is 0, so that a Q is 0 for +inf; -inf
+  // and the derivative of both infinities are NaN, as in the erf form
+  const float2 a = make_float2(fmaxf(-v.x, fminf(v.x, 64.0f)), fmaxf(-v.y, fminf(v.y, 64.0f)));
   const float2 u = __ffma2_rn(make_float2(fminf(a.x, 6.0f), fminf(a.y, 6.0f)),
                               make_float2(1.0f / 3.0f, 1.0f / 3.0f), make_float2(-1.0f, -1.0f));
   float2 p = make_float2(c[GELU_T_DEG], c[GELU_T_DEG]);
@@ -185,10 +186,10 @@ __device__ __forceinline__ void tr_gelu2(float2 v, float2* g, float2* d) {
   float2 h;
   asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(h.x) : "f"(v.x));
   asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(h.y) : "f"(v.y));
-  const float2 na = make_float2(-a.x, -a.y);
-  if (g) *g = __ffma2_rn(na, __fmul2_rn(e, p), h);
+  if (g) *g = __ffma2_rn(make_float2(-a.x, -a.y), __fmul2_rn(e, p), h);
   if (d) {
-    const float2 r = __fmul2_rn(e, __ffma2_rn(na, make_float2(0.39894228040143268f, 0.39894228040143268f), p));
+    const float2 nv = make_float2(-fabsf(v.x), -fabsf(v.y));
+    const float2 r = __fmul2_rn(e, __ffma2_rn(nv, make_float2(0.39894228040143268f, 0.39894228040143268f), p));
     // a NaN compares false with both: v itself
     *d = make_float2(v.x >= 0.0f ? 1.0f - r.x : (v.x < 0.0f ? r.x : v.x),
                      v.y >= 0.0f ? 1.0f - r.y : (v.y < 0.0f ? r.y : v.y));
