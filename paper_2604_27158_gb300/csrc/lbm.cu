@@ -738,7 +738,28 @@ __global__ void __launch_bounds__(32 * kChunkRows) k_copy_chunk(const GridDev* _
     *reinterpret_cast<float4*>(dir == 0 ? s + i * plane : c + i * cells) = v[i];
 }
 
-// Moments of the pulled level (198 -> 103 us on 8.4 M cells; HBM needs 59: the unstaged loads of
+// Moments of the pulled level, one cell a thread: for batches that leave multiprocessors idle, where
+// a lane's four cells one after the other are four times the wait.
+__global__ void __launch_bounds__(kBlock) k_macro_cell(const GridDev* __restrict__ grids,
+                                                       int ngrids,
+                                                       const uint32_t* __restrict__ mask,
+                                                       const float* __restrict__ src,
+                                                       float* __restrict__ rho_o,
+                                                       float* __restrict__ ux_o,
+                                                       float* __restrict__ uy_o) {
+  int gidx, x, y;
+  if (!cell_of_thread(grids, ngrids, gidx, x, y)) return;
+  const GridDev G = grids[gidx];  // registers: stores below cannot alias it
+  float g[kQ];
+  float rho = 1.0f, ux = 0.0f, uy = 0.0f, drho;
+  if (pull_cell(G, mask, src, x, y, g)) moments(G, g, drho, rho, ux, uy);
+  const long long c = G.cell_off + (long long)y * G.nx + x;
+  if (rho_o) rho_o[c] = rho;
+  if (ux_o) ux_o[c] = ux;
+  if (uy_o) uy_o[c] = uy;
+}
+
+// ... a chunk a lane (198 -> 103 us on 8.4 M cells; HBM needs 59: the unstaged loads of
 // a warp's one row leave gaps).
 __global__ void __launch_bounds__(32 * kChunkRows) k_macro(const GridDev* __restrict__ grids,
                                                           const int4* __restrict__ tiles,
@@ -1279,8 +1300,12 @@ int lbm_step(lbm_handle* h, int nsteps, void* stream) {
 int lbm_macro(lbm_handle* h, float* rho_d, float* ux_d, float* uy_d, void* stream) {
   LBM_REQUIRE(h != nullptr, "lbm_macro: null handle");
   const int out_vec = aligned16(rho_d) && aligned16(ux_d) && aligned16(uy_d);
-  k_macro<<<h->ntiles_v[kChunkVariant], 32 * kChunkRows, 0, S(stream)>>>(
-      h->gd_d, h->tiles_d[kChunkVariant], h->mask, h->f[h->cur], rho_d, ux_d, uy_d, out_vec);
+  if (chunk_pays(h))
+    k_macro<<<h->ntiles_v[kChunkVariant], 32 * kChunkRows, 0, S(stream)>>>(
+        h->gd_d, h->tiles_d[kChunkVariant], h->mask, h->f[h->cur], rho_d, ux_d, uy_d, out_vec);
+  else
+    k_macro_cell<<<h->nblk_total, kBlock, 0, S(stream)>>>(h->gd_d, h->ngrids, h->mask,
+                                                          h->f[h->cur], rho_d, ux_d, uy_d);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
@@ -1350,7 +1375,10 @@ int lbm_reinit_from_macro(lbm_handle* h, const float* rho_d, const float* ux_d,
 int lbm_vorticity(lbm_handle* h, const float* ux_d, const float* uy_d, float* omega_d,
                   void* stream) {
   LBM_REQUIRE(h != nullptr && ux_d && uy_d && omega_d, "lbm_vorticity: bad arguments");
-  if (h->dense4 && aligned16(ux_d) && aligned16(uy_d) && aligned16(omega_d))
+  // one small grid has no grid to search for: 2.4 us a cell a thread, 2.7 a chunk a lane on 128 x
+  // 64; fifteen grids of 64 x 31 3.2 and 2.8
+  if (h->dense4 && (h->ngrids > 1 || chunk_pays(h)) && aligned16(ux_d) && aligned16(uy_d) &&
+      aligned16(omega_d))
     k_vorticity_chunk<<<h->ntiles_v[kChunkVariant], 32 * kChunkRows, 0, S(stream)>>>(
         h->gd_d, h->tiles_d[kChunkVariant], h->mask, ux_d, uy_d, omega_d);
   else

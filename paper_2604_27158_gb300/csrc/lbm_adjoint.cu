@@ -227,8 +227,8 @@ __global__ void __launch_bounds__(kBlock) k_adj_step(const GridDev* __restrict__
   for (int i = 0; i < kQ; ++i) o[i * P + here] = l[i];
 }
 
-// k_adj_macro with a chunk of four cells a lane, for batches whose canonical and dense rows are
-// 16-byte aligned (2.1 M cells: 64 -> 38 us).  The adjoint step in this form took 86 us: both
+// k_adj_macro with a chunk of four cells a lane, for batches that fill the chip (chunk_pays) and
+// whose canonical and dense rows are 16-byte aligned (2.1 M cells: 64 -> 38 us).  The adjoint step in this form took 86 us: both
 // gathers of four cells leave too few warps, so it stays one cell a thread.
 __device__ __forceinline__ void store9_chunk(const GridDev& Gc, float* buf, const ChunkAt& at,
                                              const float v[kQ][4]) {
@@ -432,8 +432,8 @@ int lbm_adjoint_macro(lbm_handle* h, const float* gstar_d, const float* drho_d,
   LBM_REQUIRE(h != nullptr && gstar_d != nullptr && drho_d != nullptr && dux_d != nullptr &&
                   duy_d != nullptr && mu_d != nullptr,
               "lbm_adjoint_macro: null argument");
-  if (h->dense4 && aligned16(gstar_d) && aligned16(drho_d) && aligned16(dux_d) &&
-      aligned16(duy_d) && aligned16(mu_d))
+  if (h->dense4 && chunk_pays(h) && aligned16(gstar_d) && aligned16(drho_d) &&
+      aligned16(dux_d) && aligned16(duy_d) && aligned16(mu_d))
     k_adj_macro_chunk<<<h->ntiles_v[kChunkVariant], 32 * kChunkRows, 0, AS(stream)>>>(
         h->gd_d, h->tiles_d[kChunkVariant], h->mask, gstar_d, drho_d, dux_d, duy_d, mu_d);
   else

@@ -54,6 +54,11 @@ int residual_step(Handle* h, double* out_h, int update_prev, cudaStream_t s);
 constexpr int kReinitRows = 6;
 // The chunk kernels (lbm_chunk.cuh) take the tile table of shape kChunkVariant (4 rows).
 constexpr int kChunkVariant = 1;
+// Moments and their adjoint take a chunk a lane once the batch fills the chip with one cell a thread,
+// 1024 threads a multiprocessor: up to there only latency counts, and a lane's four cells are the
+// longer chain.  Cell against chunk, us: 128 x 64 2.6 : 4.0 (adjoint 3.0 : 4.6), nine grids of 128^2
+// 4.4 : 4.5 (5.1 : 5.4), ten 5.7 : 4.6 (6.7 : 5.7), eight of 256^2 10.3 : 5.8 (12.5 : 7.5).
+inline bool chunk_pays(const Handle* h) { return h->layout.cells > (size_t)1024 * h->nsm; }
 int reinit_init(Handle* h);  // sets the kernel's shared-memory limit (once per handle)
 int reinit_launch(Handle* h, const int4* tiles, int ntiles, const float* rho_d,
                   const float* ux_d, const float* uy_d, int neq_mode, cudaStream_t s);

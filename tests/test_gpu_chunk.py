@@ -68,3 +68,37 @@ def test_chunk_kernels_equal_cell_kernels(kind):
             assert float((r - want).abs().max()) < 1e-6
             assert bool((u[solid] == 0).all())
         lat.close()
+
+
+@pytest.mark.parametrize("kind", ["periodic", "pressure", "velocity"])
+def test_small_and_large_batches_agree(kind):
+    """Moments and their adjoint of small batches (a cell a thread) against the same grids beside
+    one that fills the chip (a chunk a lane, SIZES + 163,840 cells); vorticity of single grids
+    likewise.  FP32 rounding: 2e-6 of the largest."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    sizes = SIZES + [(33, 7), (127, 5), (130, 6)] if kind != "pressure" else SIZES
+    small, large = _lattice(kind, sizes, 3), _lattice(kind, sizes + [(640, 256)], 3)
+    n = small.cells
+    assert n < 100_000
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    state = 1e-2 * torch.randn(9 * large.cells, generator=gen, device="cuda")
+    fields = [0.02 * torch.randn(large.cells, generator=gen, device="cuda") for _ in range(3)]
+    small.set_state(state[:9 * n])
+    large.set_state(state)
+
+    def near(x, y):
+        return float((x - y).abs().max()) <= 2e-6 * float(y.abs().max())
+
+    for a, b in zip(small.macro(), large.macro()):
+        assert near(a, b[:n])
+    a = small.adjoint_macro(state[:9 * n], *[f[:n] for f in fields])
+    assert near(a, large.adjoint_macro(state, *fields)[:9 * n])
+    omega = large.vorticity(*fields[:2])
+    for k, w in enumerate(large.split(omega)[:len(sizes)]):
+        one = Lattice([large.grids[k]], [large.solid[k]], u_max=0.9)
+        u = [large.split(f)[k].reshape(-1).contiguous() for f in fields[:2]]
+        assert torch.equal(one.vorticity(*u), w.reshape(-1))
+        one.close()
+    small.close()
+    large.close()
