@@ -737,7 +737,7 @@ void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks) {
 // warp copies its wrapped cells one by one, so its tasks end last, and rows up to two warps long
 // have no other warps to hide it; with a body force, whose collision is longer, longer rows lose
 // as well.  Measured against single steps: 0.89 to 1.11 of the speed on 1 .. 50 grids of 33 ..
-// 230 columns; from 256 columns on 1.0 to 1.3 without a force, 0.78 to 1.07 with one.  So a
+// 230 columns; from 256 columns on 0.98 to 1.3 without a force, 0.78 to 1.07 with one.  So a
 // batch most of whose cells lie in such rows steps singly.
 bool sweep_pays(const std::vector<GridDev>& gd) {
   long long narrow = 0, all = 0;
