@@ -1082,7 +1082,7 @@ def main():
         }
         # our kernels per step: FNO on the tensor-core path (table kernel + lift + 5 per
         # layer + decoder, else 2 twiddle + lift + 5 per layer + decoder), reinit, fill,
-        # pack/unpack, one pass kernel per two LBM steps (a step kernel for the odd one out),
+        # pack/unpack, two pass kernels per four LBM steps (a step kernel for each one left over),
         # per check the step kernel with statistics (the last check's step is computed and
         # not kept) and two reduction kernels
         fno_k = (1 + 1 + 5 * 4 + 1) if net.uses_tensor_cores(NY, NX) else (2 + 1 + 5 * 4 + 1)
@@ -1090,7 +1090,7 @@ def main():
         lbm_k, done = 0, 0
         for c in range(checks):  # a check's step opens the next interval
             n = min(CHECK_EVERY, steps_per_solve - done) - (1 if c else 0)
-            lbm_k += n // STEPS_PER_PASS + n % STEPS_PER_PASS
+            lbm_k += n - n // 4 * 4 // STEPS_PER_PASS  # four steps at a time are two passes
             done = min(done + CHECK_EVERY, steps_per_solve)
         per_step = fno_k + 1 + 1 + 2 + lbm_k + 3 * checks
         line["gpu_launches"] = per_step * args.steps

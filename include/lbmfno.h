@@ -104,8 +104,11 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
 
 /* Advance every grid by nsteps fused collide+stream steps (Sec. 2.1 loop:
  * equilibrium, SRT collision, streaming with halfway bounce-back, moments).
- * One kernel launch per two steps (a pass over the populations that takes both), and
- * one for a last odd step; bitwise equal to single steps. */
+ * Batches that gain from it take four steps at a time as two passes over the
+ * populations, two steps and one kernel launch each; the rest, and other batches, one
+ * launch per step.  Bitwise equal to single steps.  A call with an even nsteps leaves the
+ * state in the buffer it found it in (an odd one in the other), so a CUDA graph that
+ * captured it may be replayed, and may alternate with other calls of even nsteps. */
 int lbm_step(lbm_handle* h, int nsteps, void* stream);
 
 /*

@@ -189,7 +189,6 @@ struct hybrid_handle {
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   cudaEvent_t ev_fno = nullptr;   // start of an FNO step (the groups' branches wait on it)
   cudaGraphExec_t cycle[2] = {nullptr, nullptr};  // by starting buffer parity
-  int cycle_end[2] = {0, 0};                      // buffer a cycle leaves the state in
 };
 
 static inline cudaStream_t HS(void* s) { return reinterpret_cast<cudaStream_t>(s); }
@@ -423,12 +422,11 @@ int hybrid_advance(hybrid_handle* h, int cycles, hybrid_stats* out_h, int64_t* g
         LBM_CHECK_CUDA(ec);
         LBM_CHECK_CUDA(cudaGraphInstantiate(&h->cycle[parity], g, 0));
         cudaGraphDestroy(g);
-        h->cycle_end[parity] = L->cur;
         L->cur = parity;  // capture recorded the launches without running them
         L->steps = steps_before;
       }
       LBM_CHECK_CUDA(cudaGraphLaunch(h->cycle[parity], h->cap));
-      L->cur = h->cycle_end[parity];
+      if (c.k_lbm % 2) L->cur ^= 1;
       L->steps = 0;  // the cycle ends with a re-initialisation
       stats.steps += c.k_lbm;
       stats.fno_calls += c.m_fno * (int)h->groups.size() * (h->fno_u ? 2 : 1);

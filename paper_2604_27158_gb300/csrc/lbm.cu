@@ -1284,12 +1284,16 @@ int lbm_step(lbm_handle* h, int nsteps, void* stream) {
     h->steps += nsteps;
     return LBM_OK;
   }
-  int left = nsteps;
-  for (; h->sweep && left >= kSweepSteps; left -= kSweepSteps) {
+  // A caller's CUDA graph holds the buffers of the calls it captured: it can be replayed when the
+  // state ends in the buffer it started from, as nsteps single steps leave it for an even nsteps.
+  // So passes, one switch of the buffers for two steps, come in pairs.
+  static_assert(kSweepSteps == 2, "a pair of passes switches the buffers as often as its steps, modulo 2");
+  const int passes = h->sweep ? nsteps / (2 * kSweepSteps) * 2 : 0;
+  for (int k = 0; k < passes; ++k) {
     LBM_TRY(sweep_launch(h, h->f[h->cur], h->f[h->cur ^ 1], s));
     h->cur ^= 1;
   }
-  for (; left > 0; --left) {
+  for (int k = kSweepSteps * passes; k < nsteps; ++k) {
     LBM_TRY(launch_step(h, h->variant, kModeStep, h->f[h->cur], h->f[h->cur ^ 1], s));
     h->cur ^= 1;
   }
