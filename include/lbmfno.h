@@ -414,8 +414,8 @@ int fno_train_query(const fno_config* cfg_h, int B, int H, int W, fno_train_size
 
 /* out_d [B][c_out][H][W] = FNO(in_d [B][c_in][H][W]); the input is used as given
  * (no bfloat16 rounding), the coordinate channels as in fno_forward.  saved_d:
- * saved_bytes, kept unchanged until the matching backward; ws_d: ws_bytes,
- * 256-byte aligned.  Parameters are read, not kept. */
+ * saved_bytes, 8-byte aligned (16-byte aligned is faster), kept unchanged until the
+ * matching backward; ws_d: ws_bytes, 256-byte aligned.  Parameters are read, not kept. */
 int fno_train_forward(const fno_config* cfg_h, const float* params_d, const float* in_d,
                       float* out_d, int B, int H, int W, float* saved_d, void* ws_d,
                       void* stream);

@@ -350,6 +350,7 @@ struct PwArgs {
   float* out;
   size_t P, hw;
   int cin, cout, trans, in_act, out_act, act, planar;
+  int in_vec, out_vec;  // pixels of `in`, and of every array of cout channels, are whole 16-byte units
   int W, m, ep;      // row length; modes and table pitch (z)
   int ap, wp, zp;    // row pitches: inputs, weights, coefficients
   int ntiles, tpr;   // tiles; tiles a row (z)
@@ -390,7 +391,7 @@ __global__ void __launch_bounds__(NT, pw_ctas(NT)) k_tr_pw(const PwArgs a) {
     }
   };
   // items of a pixel's inputs as they are copied: four channels, or one
-  const bool quad = (cin & 3) == 0;
+  const bool quad = a.in_vec;
   const Walk wa(NT, quad ? cin >> 2 : cin), we(NT, max(a.m, 1)),
       wz(NT, cout);
   auto load = [&](int t, int buf, bool zrow) {
@@ -497,7 +498,7 @@ __global__ void __launch_bounds__(NT, pw_ctas(NT)) k_tr_pw(const PwArgs a) {
             if (og * 4 + j < cout) a.out[(b * cout + og * 4 + j) * a.hw + q] = v[j];
         } else {
           // derivative of the activation (pre) or of the one whose argument dz holds, and value
-          const bool quad_out = (cout & 3) == 0;
+          const bool quad_out = a.out_vec;
           float2 w0 = make_float2(v[0], v[1]), w1 = make_float2(v[2], v[3]);
           float2 f0 = w0, f1 = w1;
           if (a.dz || a.d) {
@@ -561,10 +562,11 @@ struct WgArgs {
   float* part;
   size_t P;
   int cout, cin, in_act, act;
+  int dz_vec, in_vec;  // pixels are whole 16-byte units
 };
-__device__ __forceinline__ void wg_load(const float* src, int n, int c, int pitch, float* dst,
-                                        const Walk& from) {
-  if ((c & 3) == 0) {
+__device__ __forceinline__ void wg_load(const float* src, int n, int c, int vec, int pitch,
+                                        float* dst, const Walk& from) {
+  if (vec) {
     for (Walk w = from; w.r < n; w.next()) cpa16(dst + w.r * pitch + 4 * w.c, src + w.r * c + 4 * w.c);
   } else {
     for (Walk w = from; w.r < n; w.next()) cpa4(dst + w.r * pitch + w.c, src + w.r * c + w.c);
@@ -585,13 +587,13 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_tr_wgrad(const WgArgs a) {
   __syncthreads();
   const size_t tiles = (a.P + kWgTile - 1) / kWgTile;
   const size_t ta = tiles * blockIdx.x / gridDim.x, tb = tiles * (blockIdx.x + 1) / gridDim.x;
-  const Walk wd(kWgThreads, (a.cout & 3) ? a.cout : a.cout >> 2),
-      wi(kWgThreads, (a.cin & 3) ? a.cin : a.cin >> 2);
+  const Walk wd(kWgThreads, a.dz_vec ? a.cout >> 2 : a.cout),
+      wi(kWgThreads, a.in_vec ? a.cin >> 2 : a.cin);
   auto load = [&](size_t t, float* st) {
     const size_t p0 = t * kWgTile;
     const int n = (int)min((size_t)kWgTile, a.P - p0);
-    wg_load(a.dz + p0 * a.cout, n, a.cout, dp, st, wd);
-    wg_load(a.in + p0 * a.cin, n, a.cin, ip, st + kWgTile * dp, wi);
+    wg_load(a.dz + p0 * a.cout, n, a.cout, a.dz_vec, dp, st, wd);
+    wg_load(a.in + p0 * a.cin, n, a.cin, a.in_vec, ip, st + kWgTile * dp, wi);
   };
   float2 acc[8][4];
   float db = 0.0f;
@@ -709,7 +711,7 @@ __global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f
                                                      float2* __restrict__ x1,
                                                      const float* __restrict__ ex, size_t rows,
                                                      int W, int C, int cp, int m, int ng, int ks,
-                                                     int ep) {
+                                                     int ep, int vec) {
   extern __shared__ __align__(16) float sm[];
   const int stage = kDftX * (kDftM + ep);
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -718,7 +720,7 @@ __global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f
   const size_t row0 = (size_t)blockIdx.x * rpb;
   const int nr = (int)min((size_t)rpb, rows - row0);
   const int nthr = blockDim.x;
-  const bool quad = (C & 3) == 0;
+  const bool quad = vec;
   const Walk wf(nthr, quad ? C >> 2 : C);
   auto load = [&](int x0, float* st) {
     const int n = min(kDftX, W - x0);
@@ -797,7 +799,7 @@ __global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f
 __global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
                                                   float2* __restrict__ xh,
                                                   const float4* __restrict__ ey, int H, int W,
-                                                  int C, int m, int adjoint_scale) {
+                                                  int C, int m, int adjoint_scale, int vec) {
   __shared__ float4 es[kDftYC][kDftYA];
   __shared__ float4 red[kDftYA][32];
   const int b = blockIdx.x / m, kx = blockIdx.x % m, a0 = blockIdx.y * kDftYA;
@@ -846,8 +848,13 @@ __global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
   const int a = wp;  // kDftYA == 8 warps
   if (on && a0 + a < 2 * m) {
     const float4 r = red[a][lane];
-    *reinterpret_cast<float4*>(xh + (((size_t)b * 2 * m + a0 + a) * m + kx) * C + 2 * lane) =
-        make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sc);
+    float2* o = xh + (((size_t)b * 2 * m + a0 + a) * m + kx) * C + 2 * lane;
+    if (vec) {
+      *reinterpret_cast<float4*>(o) = make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sc);
+    } else {
+      o[0] = make_float2(r.x * sc, r.y * sc);
+      o[1] = make_float2(r.z * sc, r.w * sc);
+    }
   }
 }
 
@@ -1257,6 +1264,12 @@ struct TrCtx {
   unsigned char* ws;
 };
 
+// Whether pixels of c channels at p are whole 16-byte units: the caller's saved_d may be 8-byte
+// aligned only, and its arrays are then copied a value at a time.
+int vec_of(const void* p, int c) {
+  return c % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+}
+
 // A row pitch of at least n floats: an odd number of 16-byte units.
 int odd_pitch(int n) { return 4 * (((n + 3) / 4) | 1); }
 constexpr size_t kPwSmemMax = 227u << 10;
@@ -1314,6 +1327,8 @@ int pw(const TrCtx& x, const float* in, int cin, const float* w, int trans, cons
   a.out_act = o.out_act;
   a.act = x.c->activation;
   a.planar = o.planar;
+  a.in_vec = vec_of(in, cin);
+  a.out_vec = vec_of(out, cout) && vec_of(o.d, cout) && vec_of(o.dz, cout) && vec_of(o.pre, cout);
   a.W = x.W;
   a.m = x.c->modes;
   a.ep = x.pl.ep;
@@ -1335,7 +1350,8 @@ size_t wg_smem(int cout, int cin) {
 int wgrad(const TrCtx& x, const float* dz, int cout, const float* in, int cin, int in_act,
           float* dw, float* db) {
   float* part = reinterpret_cast<float*>(x.ws + x.pl.part);
-  const WgArgs a{dz, in, part, x.pl.P, cout, cin, in_act, x.c->activation};
+  const WgArgs a{dz, in, part, x.pl.P, cout, cin, in_act, x.c->activation, vec_of(dz, cout),
+                 vec_of(in, cin)};
   k_tr_wgrad<<<x.pl.wg_blocks, kWgThreads, wg_smem(cout, cin), x.st>>>(a);
   LBM_CHECK_LAUNCH();
   k_tr_wgrad_reduce<<<nb((size_t)cout * (cin + 1), 32), 256, 0, x.st>>>(part, x.pl.wg_blocks, cout,
@@ -1357,10 +1373,12 @@ int spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_scale)
   auto kernel = np == 4 ? k_tr_dft_x<4> : (np == 6 ? k_tr_dft_x<6> : (np == 7 ? k_tr_dft_x<7>
                                                                               : k_tr_dft_x<8>));
   kernel<<<nb(rows, kDftM / cp), 32 * ng * ks, dft_x_smem(ep, np, ng), x.st>>>(
-      f, x1, reinterpret_cast<const float*>(x.ws + x.pl.ex), rows, x.W, C, cp, m, ng, ks, ep);
+      f, x1, reinterpret_cast<const float*>(x.ws + x.pl.ex), rows, x.W, C, cp, m, ng, ks, ep,
+      vec_of(f, C));
   LBM_CHECK_LAUNCH();
   k_tr_dft_y<<<dim3(x.B * m, nb(2 * m, kDftYA)), 256, 0, x.st>>>(
-      x1, out, reinterpret_cast<const float4*>(x.ws + x.pl.ey), x.H, x.W, C, m, adjoint_scale);
+      x1, out, reinterpret_cast<const float4*>(x.ws + x.pl.ey), x.H, x.W, C, m, adjoint_scale,
+      vec_of(out, 4));
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
@@ -1498,14 +1516,16 @@ int set_smem_limits() {
   return LBM_OK;
 }
 
-int tr_setup(const fno_config* cfg, const float* params, int B, int H, int W, void* ws,
-             void* stream, TrCtx* x) {
+int tr_setup(const fno_config* cfg, const float* params, const float* saved, int B, int H, int W,
+             void* ws, void* stream, TrCtx* x) {
   LBM_REQUIRE(cfg != nullptr && params != nullptr && ws != nullptr, "fno_train: null argument");
   LBM_TRY(tr_offsets(*cfg, &x->off));
   LBM_REQUIRE(B >= 1 && H >= 2 && W >= 2 && H <= 8192 && W <= 2048,
               "fno_train: need B >= 1, 2 <= H <= 8192, 2 <= W <= 2048");
   LBM_REQUIRE(2 * cfg->modes <= H && cfg->modes <= W / 2, "fno_train: need 2m <= H and m <= W/2");
   LBM_REQUIRE((reinterpret_cast<uintptr_t>(ws) & 255) == 0, "fno_train: ws must be 256-byte aligned");
+  LBM_REQUIRE((reinterpret_cast<uintptr_t>(saved) & 7) == 0,
+              "fno_train: saved_d must be 8-byte aligned");
   LBM_TRY(set_smem_limits());
   x->c = cfg;
   x->pl = tr_plan(*cfg, B, H, W);
@@ -1562,7 +1582,7 @@ int fno_train_forward(const fno_config* cfg_h, const float* params_d, const floa
   LBM_REQUIRE(in_d != nullptr && out_d != nullptr && saved_d != nullptr,
               "fno_train_forward: null argument");
   TrCtx x;
-  LBM_TRY(tr_setup(cfg_h, params_d, B, H, W, ws_d, stream, &x));
+  LBM_TRY(tr_setup(cfg_h, params_d, saved_d, B, H, W, ws_d, stream, &x));
   const fno_config& c = *cfg_h;
   const TrPlan& pl = x.pl;
   const TrOff& o = x.off;
@@ -1613,7 +1633,7 @@ int fno_train_backward(const fno_config* cfg_h, const float* params_d, const flo
   LBM_REQUIRE(dout_d != nullptr && saved_d != nullptr && dparams_d != nullptr,
               "fno_train_backward: null argument");
   TrCtx x;
-  LBM_TRY(tr_setup(cfg_h, params_d, B, H, W, ws_d, stream, &x));
+  LBM_TRY(tr_setup(cfg_h, params_d, saved_d, B, H, W, ws_d, stream, &x));
   const fno_config& c = *cfg_h;
   const TrPlan& pl = x.pl;
   const TrOff& o = x.off;

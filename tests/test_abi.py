@@ -116,3 +116,16 @@ def test_hybrid_workspace_holds_every_group_and_network():
     assert ws(one) >= fno_ws[(3, 64, 128)]
     assert ws(two) - ws(one) >= fno_ws[(2, 48, 96)]
     assert ws(two) >= sum(fno_ws.values())
+
+
+@pytest.mark.parametrize("act", [0, 1])
+def test_training_refuses_misaligned_saved_activations(act):
+    """saved_d holds complex pairs: a buffer that is not 8-byte aligned is refused on the host,
+    by either call, before anything is launched (the pointers here are never read)."""
+    from paper_2604_27158_gb300.fno import FnoShape
+    cfg = FnoShape(width=8, layers=1, modes=2, dec_size=8, activation=act).c()
+    lib, p = _abi.lib(), 4096
+    for off in (1, 4, 12):
+        assert lib.fno_train_forward(ctypes.byref(cfg), p, p, p, 1, 8, 8, p + off, p, None) == _abi.LBM_ERR_INVALID_ARG
+        assert lib.fno_train_backward(ctypes.byref(cfg), p, p, p + off, p, None, 1, 8, 8, p,
+                                      None) == _abi.LBM_ERR_INVALID_ARG
