@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(NT, pw_ctas(NT)) k_tr_pw(const PwArgs a) {
 // (o, cin) of the partial is db).  Block k covers a contiguous range of pixel tiles; a thread
 // owns 8 x 8 pairs (two quads along each axis) and one pixel in `groups`, the groups' sums are
 // added in order at the end.  FP32 multiply-adds bound it (32 packed ones for four shared loads);
-// stages are copied two ahead of use.
+// stages are copied one ahead of use.
 struct WgArgs {
   const float* dz;
   const float* in;
@@ -646,30 +646,45 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_tr_wgrad(const WgArgs a) {
   }
   cpa_wait<0>();
   __syncthreads();
-  // the groups' sums, in order
+  // The groups' sums, in order: as many groups at a time as the stages' memory holds write their
+  // accumulators, then each pair's are added by one thread.  (One group after the other, a
+  // barrier each, took 85 of 93 us on layers of 8 x 8 channels, which have 64 groups.)
   float* red = sm;  // [dp][ip + 1]
   const int rp = ip + 1;
+  float* slot = sm + (dp * rp + 1) / 2 * 2;  // [nslot][dp][ip]
+  const int nslot = (2 * stage - (dp * rp + 1)) / (dp * ip), have = min(groups, kWgTile);
   for (int j = threadIdx.x; j < dp * rp; j += kWgThreads) red[j] = 0.0f;
-  __syncthreads();
-  for (int q = 0; q < groups; ++q) {
-    if (g == q) {
+  for (int q = 0; q < have; q += nslot) {
+    __syncthreads();
+    if (g >= q && g < min(q + nslot, have)) {
+      float* to = slot + (g - q) * dp * ip;
 #pragma unroll
       for (int o = 0; o < 8; ++o) {
         const int oo = (o >> 2) * nto * 4 + og * 4 + (o & 3);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int ii = (i >> 1) * nti * 4 + ig * 4 + (i & 1) * 2;
-          red[oo * rp + ii] += acc[o][i].x;
-          red[oo * rp + ii + 1] += acc[o][i].y;
-        }
+        for (int i = 0; i < 4; ++i)
+          *reinterpret_cast<float2*>(to + oo * ip + (i >> 1) * nti * 4 + ig * 4 + (i & 1) * 2) =
+              acc[o][i];
       }
     }
     __syncthreads();
+    const int n = min(nslot, have - q);
+    for (int j = threadIdx.x; j < dp * ip; j += kWgThreads) {
+      const int oo = j / ip;
+      float v = red[oo * rp + j - oo * ip];
+      for (int k = 0; k < n; ++k) v += slot[k * dp * ip + j];
+      red[oo * rp + j - oo * ip] = v;
+    }
   }
-  for (int q = 0; q < nbs; ++q) {
-    if (bs == q) red[bo * rp + ip] += db;
-    __syncthreads();
+  __syncthreads();
+  if (bs < nbs) slot[bs * dp + bo] = db;
+  __syncthreads();
+  if (threadIdx.x < dp) {
+    float v = 0.0f;
+    for (int q = 0; q < nbs; ++q) v += slot[q * dp + threadIdx.x];
+    red[threadIdx.x * rp + ip] = v;
   }
+  __syncthreads();
   float* out = a.part + (size_t)blockIdx.x * npairs;
   for (int j = threadIdx.x; j < npairs; j += kWgThreads) {
     const int o = j / (a.cin + 1), i = j - o * (a.cin + 1);
