@@ -226,20 +226,29 @@ int lbm_get_state(lbm_handle* h, float* gstar_d, void* stream);
 int lbm_stream_probe(lbm_handle* h, int variant, void* stream);
 
 /*
- * Step-kernel tile shapes.  The fused step runs as a persistent kernel whose
- * tile shape (rows per tile, shared-memory stages, CTAs per SM) is one of
- * LBM_STEP_VARIANTS compiled shapes; all shapes give bitwise identical results.
- * lbm_autotune times every shape `reps` times on this batch (reading the
- * current state, writing only the scratch buffer: the state is unchanged),
- * selects the fastest, and optionally returns the per-shape milliseconds per
- * step (ms_h, LBM_STEP_VARIANTS entries, INFINITY for shapes that do not fit)
- * and the chosen index.  Synchronises `stream`.
+ * Step-kernel tile shapes.  The fused single step (single steps of lbm_step, steps with
+ * statistics, the persistent launch) runs as a persistent kernel whose tile shape (rows per
+ * tile, shared-memory stages, CTAs per SM) is one of LBM_STEP_VARIANTS compiled shapes; all
+ * shapes give bitwise identical results.  lbm_autotune times every shape `reps` times on
+ * this batch (reading the current state, writing only the scratch buffer: the state is
+ * unchanged), selects the fastest, and optionally returns the per-shape milliseconds per
+ * step (ms_h, LBM_STEP_VARIANTS entries, INFINITY for shapes that do not fit) and the
+ * chosen index.  It then times two single steps of that shape against one pass over two
+ * steps, and lbm_step takes passes if they are faster (before: if the estimate of
+ * lbm_query_passes says so).  Synchronises `stream`.
  */
 #define LBM_STEP_VARIANTS 6
 int lbm_autotune(lbm_handle* h, int reps, float* ms_h, int* chosen_h, void* stream);
 int lbm_set_step_variant(lbm_handle* h, int variant);
 int lbm_get_step_variant(const lbm_handle* h, int* variant_h, int* rows_per_tile_h, int* stages_h,
                          int* ctas_per_sm_h);
+
+/* Whether lbm_step takes two steps a pass where it may: the estimate for a batch that
+ * lbm_init starts with (host only), and a handle's setting (lbm_autotune replaces it by what
+ * it measures).  Results do not depend on it. */
+int lbm_query_passes(const lbm_grid* grids_h, int ngrids, int* on_h);
+int lbm_set_passes(lbm_handle* h, int on);
+int lbm_get_passes(const lbm_handle* h, int* on_h);
 
 /* Number of lbm_step time steps taken since lbm_init / the last reinit. */
 int lbm_steps_done(const lbm_handle* h, long long* out_h);

@@ -99,6 +99,9 @@ _PROTOS = {
     "lbm_get_state": ([VP, VP, VP], I),
     "lbm_steps_done": ([VP, ctypes.POINTER(ctypes.c_longlong)], I),
     "lbm_autotune": ([VP, I, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(I), VP], I),
+    "lbm_query_passes": ([ctypes.POINTER(lbm_grid), I, ctypes.POINTER(I)], I),
+    "lbm_set_passes": ([VP, I], I),
+    "lbm_get_passes": ([VP, ctypes.POINTER(I)], I),
     "lbm_set_step_variant": ([VP, I], I),
     "lbm_get_step_variant": ([VP, ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(I),
                               ctypes.POINTER(I)], I),

@@ -921,6 +921,7 @@ __global__ void __launch_bounds__(32 * kChunkRows) k_vorticity_chunk(
 struct WsPlan {
   size_t grids_off, uprev_off, seg_off, partial_off, stats_off, status_off, bar_off, tiles_off,
       sweep_off, total;
+  bool passes;  // what sweep_pays estimates
 };
 
 // Scratch of one statistics evaluation: FP32 row-segment partials, FP64 block sums,
@@ -1029,6 +1030,14 @@ static int plan_layout(const lbm_grid* grids, int ngrids, lbm_layout* lay,
   std::vector<SweepTask> sweep;
   sweep_plan(all, &sweep);
   w.total = align_up(w.sweep_off + sweep.size() * sizeof(SweepTask), 256);
+  bool one_wave = false;
+  for (int v = 0; v < LBM_STEP_VARIANTS; ++v) {
+    size_t n = 0;
+    for (const GridDev& d : all)
+      n += (size_t)d.nseg * ((d.ny + kStepVariants[v].ty - 1) / kStepVariants[v].ty);
+    one_wave = one_wave || n <= (size_t)kSweepSms * kStepVariants[v].minb;
+  }
+  w.passes = sweep_pays(all, sweep, one_wave);
   lay->f_elems = (size_t)kQ * plane_all;
   lay->mask_words = words;
   lay->cells = cells;
@@ -1172,6 +1181,15 @@ int lbm_query_layout(const lbm_grid* grids_h, int ngrids, lbm_layout* out_h) {
   return plan_layout(grids_h, ngrids, out_h, nullptr, nullptr);
 }
 
+int lbm_query_passes(const lbm_grid* grids_h, int ngrids, int* on_h) {
+  LBM_REQUIRE(on_h != nullptr, "lbm_query_passes: null output");
+  lbm_layout lay;
+  WsPlan wp;
+  LBM_TRY(plan_layout(grids_h, ngrids, &lay, nullptr, &wp));
+  *on_h = wp.passes;
+  return LBM_OK;
+}
+
 int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float* f_a_d,
              float* f_b_d, void* ws_d, double u_max, void* stream, lbm_handle** out) {
   LBM_REQUIRE(out != nullptr, "lbm_init: null handle output");
@@ -1224,7 +1242,7 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
   sweep_plan(h->gd, &sweep);
   h->sweep_d = reinterpret_cast<SweepTask*>(ws + wp.sweep_off);
   h->sweep_ctas = (int)(sweep.size() / kSweepWarps);
-  h->sweep = sweep_pays(h->gd);
+  h->sweep = wp.passes;
   h->stats_h.assign((size_t)ngrids * R_COUNT, 0.0);
   h->u_max2 = (float)(u_max * u_max);
   cudaStream_t s = S(stream);
@@ -1289,12 +1307,14 @@ int lbm_step(lbm_handle* h, int nsteps, void* stream) {
   // So passes, one switch of the buffers for two steps, come in pairs.
   static_assert(kSweepSteps == 2, "a pair of passes switches the buffers as often as its steps, modulo 2");
   const int passes = h->sweep ? nsteps / (2 * kSweepSteps) * 2 : 0;
-  for (int k = 0; k < passes; ++k) {
-    LBM_TRY(sweep_launch(h, h->f[h->cur], h->f[h->cur ^ 1], s));
-    h->cur ^= 1;
-  }
+  // The single steps come first: behind a pass one took 45 us longer in some tile shapes (100 uneven
+  // grids, 80 us a step).
   for (int k = kSweepSteps * passes; k < nsteps; ++k) {
     LBM_TRY(launch_step(h, h->variant, kModeStep, h->f[h->cur], h->f[h->cur ^ 1], s));
+    h->cur ^= 1;
+  }
+  for (int k = 0; k < passes; ++k) {
+    LBM_TRY(sweep_launch(h, h->f[h->cur], h->f[h->cur ^ 1], s));
     h->cur ^= 1;
   }
   h->steps += nsteps;
@@ -1459,6 +1479,25 @@ int lbm_autotune(lbm_handle* h, int reps, float* ms_h, int* chosen_h, void* stre
       best = v;
     }
   }
+  // two steps of that shape against one pass, in turn, the better of two runs each; enough launches
+  // that a run of short ones takes some 0.1 ms
+  float two_ms[2] = {INFINITY, INFINITY};
+  const int n = rc == LBM_OK ? std::max(reps, std::min(16, (int)(0.1f / best_ms))) : 0;
+  for (int k = 0; k < 4 && rc == LBM_OK; ++k) {
+    const bool pass = k & 1;
+    auto launch = [&] {
+      return pass ? sweep_launch(h, src, scratch, s) : launch_step(h, best, kModeStep, src, scratch, s);
+    };
+    float ms = INFINITY;
+    for (int w = 0; w < 2 && rc == LBM_OK; ++w) rc = launch();
+    if (rc == LBM_OK && cudaEventRecord(e0, s) != cudaSuccess) rc = LBM_ERR_CUDA;
+    for (int w = 0; w < n && rc == LBM_OK; ++w) rc = launch();
+    if (rc == LBM_OK && (cudaEventRecord(e1, s) != cudaSuccess ||
+                         cudaEventSynchronize(e1) != cudaSuccess ||
+                         cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+      rc = LBM_ERR_CUDA;
+    two_ms[pass] = std::min(two_ms[pass], ms / (float)n * (pass ? 1.0f : (float)kSweepSteps));
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != LBM_OK) {
@@ -1466,6 +1505,8 @@ int lbm_autotune(lbm_handle* h, int reps, float* ms_h, int* chosen_h, void* stre
     return rc;
   }
   h->variant = best;
+  // within 4% the setting stays (these launches read one clean buffer again and again)
+  if (fabsf(two_ms[1] - two_ms[0]) > 0.04f * two_ms[0]) h->sweep = two_ms[1] < two_ms[0];
   if (chosen_h) *chosen_h = best;
   return LBM_OK;
 }
@@ -1487,6 +1528,18 @@ int lbm_get_step_variant(const lbm_handle* h, int* variant_h, int* rows_per_tile
   if (rows_per_tile_h) *rows_per_tile_h = sv.ty;
   if (stages_h) *stages_h = sv.stages;
   if (ctas_per_sm_h) *ctas_per_sm_h = h->blocks_per_sm_v[h->variant];
+  return LBM_OK;
+}
+
+int lbm_set_passes(lbm_handle* h, int on) {
+  LBM_REQUIRE(h != nullptr, "lbm_set_passes: null handle");
+  h->sweep = on != 0;
+  return LBM_OK;
+}
+
+int lbm_get_passes(const lbm_handle* h, int* on_h) {
+  LBM_REQUIRE(h != nullptr && on_h != nullptr, "lbm_get_passes: bad arguments");
+  *on_h = h->sweep;
   return LBM_OK;
 }
 

@@ -27,7 +27,7 @@ struct Handle {
                         // aligned whenever their buffers are
   struct SweepTask* sweep_d = nullptr;  // tasks of a multi-step pass (workspace)
   int sweep_ctas = 0;
-  bool sweep = false;  // lbm_step takes passes
+  bool sweep = false;  // lbm_step takes passes where it may
   unsigned* status_d = nullptr;
   unsigned status_h = 0;
   const uint32_t* mask = nullptr;

@@ -733,21 +733,49 @@ void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks) {
   while (tasks->size() % kWarps) tasks->push_back(SweepTask{});
 }
 
-// Periodic rows of a length that is no multiple of 4 wrap inside a chunk: every row of such a
-// warp copies its wrapped cells one by one, so its tasks end last, and rows up to two warps long
-// have no other warps to hide it; with a body force, whose collision is longer, longer rows lose
-// as well.  Measured against single steps: 0.89 to 1.11 of the speed on 1 .. 50 grids of 33 ..
-// 230 columns; from 256 columns on 0.98 to 1.3 without a force, 0.78 to 1.07 with one.  So a
-// batch most of whose cells lie in such rows steps singly.
-bool sweep_pays(const std::vector<GridDev>& gd) {
-  long long narrow = 0, all = 0;
+// Estimated times in us, fitted to 1,493 batches of 2,000 to 16 M cells (24 to 8,192 columns, 1 to
+// 100 grids; periodic rows with and without a force, open rows with sparse and dense disks) with a
+// spread of 5% (step, in its fastest shape) and 6% (pass).
+//  * A single step costs its launch and then the row segments of 128 columns a multiprocessor
+//    steps, more once its tiles need a second wave.
+//  * A pass costs its launch and, a wave of CTAs, rows + 2 iterations of both levels, whose
+//    length is mostly latency: three CTAs on a multiprocessor take 1.5 times as long as one.  A
+//    force makes the collision longer, rows that wrap inside a chunk copy their cells one by one,
+//    open rows complete their ends, and rows of up to 40 columns leave three quarters of the
+//    lanes idle.
+// So passes lose where rows are just too many for one wave of one-row tasks and a single step is
+// still one wave (eight forced grids of 180 x 119: 6.4 us a step, 7.2 in passes; 20 grids of 122 x
+// 120: 7.3 and 9.3), and on many narrow or ragged rows.  Taken from an estimated gain of 4% on.
+// Of 500 other batches 439 take passes then, 10 of them at less than 0.98 of the speed of single
+// steps (0.91 the least), and 11 of the other 61 would gain more than 10%.  After lbm_autotune,
+// which times both, 457 take passes, 3 at less than 0.98 (0.96), and none would gain 2%.
+bool sweep_pays(const std::vector<GridDev>& gd, const std::vector<SweepTask>& tasks, bool one_wave) {
+  double cells = 0, segs = 0, forced = 0, ragged = 0, open = 0, narrow = 0;
   for (const GridDev& d : gd) {
-    const long long cells = (long long)d.nx * d.ny;
-    all += cells;
-    const bool forced = d.fx != 0.0f || d.fy != 0.0f;
-    if (d.periodic_x && d.nx % kV != 0 && (d.nx < 256 || forced)) narrow += cells;
+    const double c = (double)d.nx * d.ny;
+    cells += c;
+    segs += (double)d.nseg * d.ny;
+    if (d.fx != 0.0f || d.fy != 0.0f) forced += c;
+    if (d.periodic_x && d.nx % kV != 0) ragged += c;
+    if (!d.periodic_x) open += c;
+    if (d.nx <= 40) narrow += c;
   }
-  return 2 * narrow <= all;
+  forced /= cells;  // shares of the cells
+  ragged /= cells;
+  open /= cells;
+  narrow /= cells;
+  const double w = segs / kSweepSms;  // row segments a multiprocessor
+  const double step = (one_wave ? 4.79 + 0.12 * w : 3.46 + 0.22 * w) + forced * (0.45 + 0.03 * w) +
+                      0.31 * ragged;
+  int rows = 0;
+  for (const SweepTask& t : tasks) rows = std::max(rows, t.rows);
+  const int wave = kSweepSms * kCtas, ctas = (int)(tasks.size() / kWarps), full = (ctas - 1) / wave;
+  const int last = (ctas - wave * full + kSweepSms - 1) / kSweepSms;  // CTAs a multiprocessor, last wave
+  static const double base[4] = {0, 1.71, 2.32, 2.51}, force[4] = {0, 0.44, 0.73, 0.85};
+  const double kind = 0.86 * ragged + 0.44 * open + 0.41 * narrow;
+  auto iteration = [&](int k) { return base[k] + force[k] * forced + kind; };
+  const double pass = 1.56 + (rows + 2) * (full * iteration(kCtas) + iteration(last));
+  return kSweepSteps * step >= 1.04 * pass;
 }
 
 int sweep_init() {

@@ -27,7 +27,9 @@ static_assert(sizeof(SweepTask) == 40, "task table entry");
 struct Handle;
 // Tasks of a batch, kSweepWarps a CTA.  Host only, a function of the grids alone.
 void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks);
-bool sweep_pays(const std::vector<GridDev>& gd);  // whether lbm_step takes passes for a batch
+// Whether passes of these tasks are estimated to beat single steps; one_wave: a single step's tiles
+// are resident at once in some shape.  Host only.
+bool sweep_pays(const std::vector<GridDev>& gd, const std::vector<SweepTask>& tasks, bool one_wave);
 int sweep_init();
 int sweep_launch(Handle* h, const float* src, float* dst, cudaStream_t s);
 

@@ -66,6 +66,14 @@ def query_layout(grids: Sequence[GridSpec]) -> lbm_layout:
     return lay
 
 
+def query_passes(grids: Sequence[GridSpec]) -> bool:
+    """Whether a new Lattice of these grids takes two steps a pass (host-only estimate)."""
+    arr = (lbm_grid * len(grids))(*[g.c() for g in grids])
+    v = ctypes.c_int()
+    call("lbm_query_passes", arr, len(grids), ctypes.byref(v))
+    return bool(v.value)
+
+
 class Lattice:
     """A batch of D2Q9 lattices resident on one GPU (a thin owner of lbm_handle)."""
 
@@ -174,13 +182,23 @@ class Lattice:
         return out
 
     def autotune(self, reps: int = 10, stream=None):
-        """Time every compiled step-kernel tile shape on this batch and keep the fastest.
+        """Time every compiled tile shape of the single-step kernel on this batch and keep the
+        fastest, then two of its steps against one pass over two steps and keep the faster.
 
         The state is unchanged.  Returns (chosen index, milliseconds per step per shape)."""
         ms = (ctypes.c_float * _abi.LBM_STEP_VARIANTS)()
         chosen = ctypes.c_int()
         call("lbm_autotune", self._h, int(reps), ms, ctypes.byref(chosen), _stream_ptr(stream))
         return chosen.value, list(ms)
+
+    def set_passes(self, on: bool) -> None:
+        """Let step() take two steps a pass over the populations (same results), or not."""
+        call("lbm_set_passes", self._h, int(bool(on)))
+
+    def passes(self) -> bool:
+        v = ctypes.c_int()
+        call("lbm_get_passes", self._h, ctypes.byref(v))
+        return bool(v.value)
 
     def set_step_variant(self, variant: int) -> None:
         call("lbm_set_step_variant", self._h, int(variant))

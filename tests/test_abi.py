@@ -129,3 +129,26 @@ def test_training_refuses_misaligned_saved_activations(act):
         assert lib.fno_train_forward(ctypes.byref(cfg), p, p, p, 1, 8, 8, p + off, p, None) == _abi.LBM_ERR_INVALID_ARG
         assert lib.fno_train_backward(ctypes.byref(cfg), p, p, p + off, p, None, 1, 8, 8, p,
                                       None) == _abi.LBM_ERR_INVALID_ARG
+
+
+# (kind, nx, ny, grids) and the measured time of two single steps over that of one pass
+MEASURED_PASSES = [
+    ("forced", 90, 60, 31, 0.74), ("forced", 293, 219, 3, 0.77), ("forced", 55, 78, 27, 0.78),
+    ("free", 122, 120, 20, 0.78), ("free", 65, 149, 14, 0.79), ("forced", 110, 152, 16, 0.77),
+    ("free", 130, 60, 16, 0.83), ("free", 54, 67, 32, 0.83), ("forced", 130, 64, 10, 0.85),
+    ("open", 32, 128, 19, 0.76), ("open", 36, 68, 30, 0.81), ("open", 33, 65, 34, 0.86),
+    ("forced", 180, 119, 8, 0.89), ("forced", 255, 100, 22, 0.85), ("forced", 193, 156, 5, 0.88),
+    ("forced", 128, 64, 1, 1.47), ("open", 512, 256, 64, 1.7), ("open", 4096, 4096, 1, 1.5),
+    ("open", 512, 256, 20, 1.6), ("free", 128, 128, 100, 1.7), ("free", 64, 64, 1, 1.44),
+    ("forced", 256, 128, 46, 1.56), ("free", 512, 100, 23, 1.46), ("forced", 621, 273, 12, 1.14),
+    ("free", 139, 79, 87, 1.43), ("open", 262, 139, 18, 1.4), ("free", 48, 48, 1, 1.5)]
+
+
+@pytest.mark.parametrize("kind,nx,ny,n,gain", MEASURED_PASSES)
+def test_passes_are_estimated_to_pay_where_they_do(kind, nx, ny, n, gain):
+    """lbm_step takes two steps a pass by an estimate that is a function of the batch alone; at
+    batches with a clear outcome it agrees with the measurement."""
+    from paper_2604_27158_gb300.lbm import query_passes
+    kw = dict(bc_west=P.BC_PRESSURE, bc_east=P.BC_PRESSURE, west_value=1.001) if kind == "open" else {}
+    grid = GridSpec(nx, ny, 0.7, fx=1e-6 if kind == "forced" else 0.0, **kw)
+    assert query_passes([grid] * n) == (gain > 1)
