@@ -26,24 +26,11 @@ def fno_train_query(shape: FnoShape, B: int, H: int, W: int) -> fno_train_sizes:
     return out
 
 
-class _Buffers:
-    """Saved-activation and scratch buffers per (B, H, W), reused across steps."""
-
-    def __init__(self):
-        self.cache = {}
-
-    def get(self, shape: FnoShape, B, H, W, device):
-        key = (shape, B, H, W)
-        if key not in self.cache:
-            sz = fno_train_query(shape, B, H, W)
-            saved = torch.empty(sz.saved_bytes // 4, dtype=torch.float32, device=device)
-            ws = torch.empty(sz.ws_bytes + 256, dtype=torch.uint8, device=device)
-            off = (-ws.data_ptr()) % 256
-            self.cache[key] = (saved, ws[off:off + sz.ws_bytes])
-        return self.cache[key]
-
-
-_BUFFERS = _Buffers()
+def _workspace(sz: fno_train_sizes, device) -> torch.Tensor:
+    """Scratch of one call, 256-byte aligned; freed to torch's stream-ordered pool after it."""
+    ws = torch.empty(sz.ws_bytes + 256, dtype=torch.uint8, device=device)
+    off = (-ws.data_ptr()) % 256
+    return ws[off:off + sz.ws_bytes]
 
 
 class FnoTrainFn(torch.autograd.Function):
@@ -54,29 +41,33 @@ class FnoTrainFn(torch.autograd.Function):
         x = x.detach().contiguous()
         B, cin, H, W = x.shape
         assert cin == shape.c_in
-        saved, ws = _BUFFERS.get(shape, B, H, W, x.device)
+        # every call keeps its own activations: several may be waiting for their backward
+        sz = fno_train_query(shape, B, H, W)
+        saved = torch.empty(sz.saved_bytes // 4, dtype=torch.float32, device=x.device)
+        ws = _workspace(sz, x.device)
         out = torch.empty((B, shape.c_out, H, W), dtype=torch.float32, device=x.device)
         cfg = shape.c()
         call("fno_train_forward", ctypes.byref(cfg), params.data_ptr(), x.data_ptr(),
              out.data_ptr(), B, H, W, saved.data_ptr(), ws.data_ptr(), _stream_ptr(None))
-        ctx.shape, ctx.dims = shape, (B, H, W)
+        ctx.shape, ctx.dims, ctx.sizes = shape, (B, H, W), sz
         ctx.need_x = ctx.needs_input_grad[1]
-        ctx.save_for_backward(params)
-        ctx.saved_buf, ctx.ws = saved, ws
+        ctx.save_for_backward(params, saved)  # given back once the backward has run
         return out
 
     @staticmethod
     def backward(ctx, dout):
-        (params,) = ctx.saved_tensors
+        params, saved = ctx.saved_tensors
         B, H, W = ctx.dims
         shape = ctx.shape
         dparams = torch.empty_like(params)
         dx = (torch.empty((B, shape.c_in, H, W), dtype=torch.float32, device=params.device)
               if ctx.need_x else None)
         cfg = shape.c()
-        call("fno_train_backward", ctypes.byref(cfg), params.data_ptr(),
-             dout.float().contiguous().data_ptr(), ctx.saved_buf.data_ptr(), dparams.data_ptr(),
-             dx.data_ptr() if dx is not None else None, B, H, W, ctx.ws.data_ptr(),
+        dout = dout.float().contiguous()
+        ws = _workspace(ctx.sizes, params.device)
+        call("fno_train_backward", ctypes.byref(cfg), params.data_ptr(), dout.data_ptr(),
+             saved.data_ptr(), dparams.data_ptr(),
+             dx.data_ptr() if dx is not None else None, B, H, W, ws.data_ptr(),
              _stream_ptr(None))
         return dparams, dx, None
 
