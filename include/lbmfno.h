@@ -243,6 +243,10 @@ int lbm_set_step_variant(lbm_handle* h, int variant);
 int lbm_get_step_variant(const lbm_handle* h, int* variant_h, int* rows_per_tile_h, int* stages_h,
                          int* ctas_per_sm_h);
 
+/* y = 1 / x, correctly rounded, as the passes of lbm_step evaluate it (four values together;
+ * caller-owned device arrays, may alias).  For tests. */
+int lbm_reciprocal_eval(const float* x_d, float* y_d, size_t n, void* stream);
+
 /* Whether lbm_step takes two steps a pass where it may: the estimate for a batch that
  * lbm_init starts with (host only), and a handle's setting (lbm_autotune replaces it by what
  * it measures).  Results do not depend on it. */

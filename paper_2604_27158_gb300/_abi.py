@@ -99,6 +99,7 @@ _PROTOS = {
     "lbm_get_state": ([VP, VP, VP], I),
     "lbm_steps_done": ([VP, ctypes.POINTER(ctypes.c_longlong)], I),
     "lbm_autotune": ([VP, I, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(I), VP], I),
+    "lbm_reciprocal_eval": ([VP, VP, ctypes.c_size_t, VP], I),
     "lbm_query_passes": ([ctypes.POINTER(lbm_grid), I, ctypes.POINTER(I)], I),
     "lbm_set_passes": ([VP, I], I),
     "lbm_get_passes": ([VP, ctypes.POINTER(I)], I),

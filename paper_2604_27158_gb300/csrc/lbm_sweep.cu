@@ -117,7 +117,8 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, dup(
 // Correctly rounded reciprocals of a lane's values, all in [0.5, 2): the approximate
 // reciprocal (within one ulp) and one fused Newton step, which rounds correctly (Markstein,
 // "Computation of elementary functions on the IBM RISC System/6000 processor", 1990); if one
-// is outside, __frcp_rn.  Equal to __frcp_rn for every float in the range (all 2^24 checked).
+// is outside, __frcp_rn.  Equal to the correctly rounded quotient for every float in the range:
+// tests/test_gpu_reciprocal.py takes all 2^24.
 __device__ __forceinline__ void rcp_lane(const float2 rho[kH], float2 inv[kH]) {
   uint32_t far = 0;
 #pragma unroll
@@ -617,6 +618,19 @@ __global__ void __launch_bounds__(kWarps * 32, kCtas)
   }
 }
 
+// rcp_lane of n values, four (a lane's) a thread; the last thread's missing ones are 1.
+__global__ void k_rcp_eval(const float* __restrict__ x, float* __restrict__ y, size_t n) {
+  const size_t at = 4 * (blockIdx.x * (size_t)blockDim.x + threadIdx.x);
+  if (at >= n) return;
+  float v[4];
+  for (int j = 0; j < 4; ++j) v[j] = at + j < n ? x[at + j] : 1.0f;
+  const float2 rho[kH] = {make_float2(v[0], v[1]), make_float2(v[2], v[3])};
+  float2 inv[kH];
+  rcp_lane(rho, inv);
+  for (int j = 0; j < 4; ++j)
+    if (at + j < n) y[at + j] = get2(inv, j);
+}
+
 constexpr size_t kSmem =
     sizeof(float) * ((size_t)kWarps * kWarpFloats + (size_t)(kT - 1) * kRing * kWarps * kEdge);
 
@@ -808,3 +822,14 @@ int sweep_launch(Handle* h, const float* src, float* dst, cudaStream_t s) {
 }
 
 }  // namespace lbmfno
+
+using namespace lbmfno;
+
+extern "C" int lbm_reciprocal_eval(const float* x_d, float* y_d, size_t n, void* stream) {
+  LBM_REQUIRE(n == 0 || (x_d != nullptr && y_d != nullptr), "lbm_reciprocal_eval: null buffer");
+  LBM_REQUIRE(n <= (size_t)1 << 32, "lbm_reciprocal_eval: n must be at most 2^32");
+  if (n == 0) return LBM_OK;
+  k_rcp_eval<<<(unsigned)((n + 1023) / 1024), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(x_d, y_d, n);
+  LBM_CHECK_LAUNCH();
+  return LBM_OK;
+}
