@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_tr_wgrad(const WgArgs a) {
   __syncthreads();
   // The groups' sums, in order: as many groups at a time as the stages' memory holds write their
   // accumulators, then each pair's are added by one thread.  (One group after the other, a
-  // barrier each, took 85 of 93 us on layers of 8 x 8 channels, which have 64 groups.)
+  // barrier each: 93 us a launch on layers of 8 x 8 channels and 22,000 pixels, now 9.)
   float* red = sm;  // [dp][ip + 1]
   const int rp = ip + 1;
   float* slot = sm + (dp * rp + 1) / 2 * 2;  // [nslot][dp][ip]
@@ -876,10 +876,12 @@ __global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
 // ---- forward pass of ReLU networks -----------------------------------------------------------
 // ReLU's derivative jumps at 0.  Sums in another order move the pre-activations that lie within
 // rounding of 0 across it, and one pixel that changes sides changes a gradient, a sum over pixels
-// with random signs, by 1e-4 of its norm or more.  So that a ReLU network's gradients do not
-// depend on how its layers are tiled, its forward pass keeps one plain order: every sum runs
-// over its terms one after the other (the kernels below, one output a thread and term loop).  Its
-// backward pass, which takes the signs as saved, uses the tiled kernels.
+// with random signs, by 1e-4 of its norm or more, with the same error against 64 bits.  So the
+// forward pass of ReLU networks keeps the order their results have always had: every sum runs over
+// its terms one after the other (the kernels below, one output a thread and term loop).  The tiled
+// kernels do not: their packed accumulators hold pairs of terms.  (Tiles whose accumulators hold
+// pairs of outputs would keep this order; there are none yet.)  The backward pass, which takes
+// the signs as saved, uses the tiled kernels.
 constexpr int kSqPix = 128;      // pixels a block of the pointwise kernel
 constexpr int kSqThreads = 256;
 constexpr int kSqAcc = 16;       // spectral accumulators a thread
@@ -894,29 +896,24 @@ __global__ void k_sq_twiddle(float2* __restrict__ tw, int N) {
 }
 
 // Pointwise linear layer over kSqPix pixels per block:
-//   v[p][o] = add[p][o] + bias[o] + sum_i Wm(o, i) * A(in[p][i]),
-//   Wm(o, i) = trans ? w[i * cout + o] : w[o * cin + i],  A = sigma if in_act else identity;
-//   pre[p][o] = v (if pre != null);  out[p][o] = out_act ? sigma(v) : v.
+//   v[p][o] = add[p][o] + bias[o] + sum_i w[o * cin + i] * in[p][i];
+//   pre[p][o] = v (if pre != null);  out[p][o] = out_act ? max(v, 0) : v.
 __global__ void __launch_bounds__(kSqPix) k_sq_pw(const float* __restrict__ in, int cin,
-                                                  const float* __restrict__ w, int trans,
+                                                  const float* __restrict__ w,
                                                   const float* __restrict__ bias,
                                                   const float* __restrict__ add, int cout,
                                                   float* __restrict__ pre, float* __restrict__ out,
-                                                  int in_act, int out_act, int act, size_t P) {
+                                                  int out_act, size_t P) {
   extern __shared__ float sm[];
   float* ws = sm;                               // [cout][cin]
   float* is = ws + cout * cin;                  // [kSqPix][cin + 1]
   float* os = is + kSqPix * (cin + 1);          // [kSqPix][cout + 1]
   const size_t p0 = (size_t)blockIdx.x * kSqPix;
   const int np = (int)min((size_t)kSqPix, P - p0);
-  for (int j = threadIdx.x; j < cout * cin; j += kSqPix) {
-    const int o = j / cin, i = j - o * cin;
-    ws[j] = trans ? w[(size_t)i * cout + o] : w[j];
-  }
+  for (int j = threadIdx.x; j < cout * cin; j += kSqPix) ws[j] = w[j];
   for (int j = threadIdx.x; j < np * cin; j += kSqPix) {
     const int t = j / cin, i = j - t * cin;
-    const float v = in[p0 * cin + j];
-    is[t * (cin + 1) + i] = in_act ? tr_act(v, act) : v;
+    is[t * (cin + 1) + i] = in[p0 * cin + j];
   }
   for (int j = threadIdx.x; j < np * cout; j += kSqPix) {
     const int t = j / cout, o = j - t * cout;
@@ -939,7 +936,7 @@ __global__ void __launch_bounds__(kSqPix) k_sq_pw(const float* __restrict__ in, 
     const int tt = j / cout, o = j - tt * cout;
     const float v = os[tt * (cout + 1) + o];
     if (pre) pre[p0 * cout + j] = v;
-    out[p0 * cout + j] = out_act ? tr_act(v, act) : v;
+    out[p0 * cout + j] = out_act ? fmaxf(v, 0.0f) : v;
   }
 }
 
@@ -991,14 +988,12 @@ __global__ void __launch_bounds__(kSqThreads) k_sq_dft_x(const float* __restrict
   }
 }
 
-// Forward y-DFT over the kept rows: Xh[b][a][kx][c] = scale(kx) sum_y X1[b][y][kx][c]
-// e^{-2 pi i ky(a) y / H}, ky(a) = a (a < m) or H - 2m + a; scale = 1, or c_kx / (H W)
-// for the adjoint of the real inverse transform.
+// Forward y-DFT over the kept rows: Xh[b][a][kx][c] = sum_y X1[b][y][kx][c]
+// e^{-2 pi i ky(a) y / H}, ky(a) = a (a < m) or H - 2m + a.
 __global__ void __launch_bounds__(kSqThreads) k_sq_dft_y(const float2* __restrict__ x1,
                                                            float2* __restrict__ xh,
                                                            const float2* __restrict__ twy,
-                                                           int H, int W, int C, int m,
-                                                           int adjoint_scale) {
+                                                           int H, int C, int m) {
   extern __shared__ float sm[];
   float2* tw = reinterpret_cast<float2*>(sm);  // H
   float2* tile = tw + H;                        // [32][C]
@@ -1037,13 +1032,11 @@ __global__ void __launch_bounds__(kSqThreads) k_sq_dft_y(const float2* __restric
       }
     }
   }
-  const float sc = adjoint_scale ? (kx == 0 ? 1.0f : 2.0f) / ((float)H * (float)W) : 1.0f;
   if (g < G) {
 #pragma unroll
     for (int k = 0; k < kSqAcc; ++k) {
       const int a = g + k * G;
-      if (a < 2 * m)
-        xh[(((size_t)b * 2 * m + a) * m + kx) * C + c] = make_float2(acc[k].x * sc, acc[k].y * sc);
+      if (a < 2 * m) xh[(((size_t)b * 2 * m + a) * m + kx) * C + c] = acc[k];
     }
   }
 }
@@ -1082,13 +1075,12 @@ __global__ void __launch_bounds__(kSqThreads) k_sq_inv_y(const float2* __restric
   }
 }
 
-// Inverse x-DFT with real output: S[row][x][c] = scale sum_kx w(kx) Re(Z[row][kx][c]
-// e^{+2 pi i kx x / W}); w(kx) = c_kx (forward) or 1 (adjoint of the forward DFT).
+// Inverse x-DFT with real output: S[row][x][c] = scale sum_kx c_kx Re(Z[row][kx][c]
+// e^{+2 pi i kx x / W}).
 __global__ void __launch_bounds__(kSqThreads) k_sq_inv_x(const float2* __restrict__ z,
                                                            float* __restrict__ s,
                                                            const float2* __restrict__ twx,
-                                                           int W, int C, int m, float scale,
-                                                           int hermitian) {
+                                                           int W, int C, int m, float scale) {
   extern __shared__ float sm[];
   float2* tw = reinterpret_cast<float2*>(sm);  // W
   float2* zr = tw + W;                          // [m][C]
@@ -1097,7 +1089,7 @@ __global__ void __launch_bounds__(kSqThreads) k_sq_inv_x(const float2* __restric
   for (int j = threadIdx.x; j < m * C; j += kSqThreads) {
     const int kx = j / C;
     float2 v = z[row * m * C + j];
-    const float wk = (hermitian && kx > 0) ? 2.0f * scale : scale;
+    const float wk = kx > 0 ? 2.0f * scale : scale;
     zr[j] = make_float2(v.x * wk, v.y * wk);
   }
   __syncthreads();
@@ -1415,17 +1407,17 @@ size_t sq_pw_smem(int cin, int cout) {
   return sizeof(float) * ((size_t)cout * cin + (size_t)kSqPix * (cin + 1) + (size_t)kSqPix * (cout + 1));
 }
 
-int sq_pw(const TrCtx& x, const float* in, int cin, const float* w, int trans, const float* bias,
-       const float* add, int cout, float* pre, float* out, int in_act, int out_act) {
+int sq_pw(const TrCtx& x, const float* in, int cin, const float* w, const float* bias,
+          const float* add, int cout, float* pre, float* out, int out_act) {
   const size_t smem = sq_pw_smem(cin, cout);
-  k_sq_pw<<<nb(x.pl.P, kSqPix), kSqPix, smem, x.st>>>(in, cin, w, trans, bias, add, cout, pre, out,
-                                                      in_act, out_act, x.c->activation, x.pl.P);
+  k_sq_pw<<<nb(x.pl.P, kSqPix), kSqPix, smem, x.st>>>(in, cin, w, bias, add, cout, pre, out,
+                                                      out_act, x.pl.P);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
 
-// X (or the adjoint-scaled dY) of a field: forward x-DFT then y-DFT over the kept rows.
-int sq_spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_scale) {
+// X of a field: forward x-DFT then y-DFT over the kept rows.
+int sq_spectral_fwd(const TrCtx& x, const float* f, float2* out) {
   const int C = x.c->width, m = x.c->modes;
   float2* x1 = reinterpret_cast<float2*>(x.ws + x.pl.x1);
   const float2* twx = reinterpret_cast<const float2*>(x.ws + x.pl.twx);
@@ -1434,13 +1426,13 @@ int sq_spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_sca
                                                                                     C, m);
   LBM_CHECK_LAUNCH();
   k_sq_dft_y<<<x.B * m, kSqThreads, (x.H + 32 * C) * sizeof(float2), x.st>>>(
-      x1, out, twy, x.H, x.W, C, m, adjoint_scale);
+      x1, out, twy, x.H, C, m);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
 
 // Real field from kept coefficients: inverse y-DFT then inverse x-DFT.
-int sq_spectral_inv(const TrCtx& x, const float2* coef, float* s, float scale, int hermitian) {
+int sq_spectral_inv(const TrCtx& x, const float2* coef, float* s, float scale) {
   const int C = x.c->width, m = x.c->modes;
   float2* z = reinterpret_cast<float2*>(x.ws + x.pl.z);
   const float2* twx = reinterpret_cast<const float2*>(x.ws + x.pl.twx);
@@ -1449,7 +1441,7 @@ int sq_spectral_inv(const TrCtx& x, const float2* coef, float* s, float scale, i
                                                                                   x.H, C, m);
   LBM_CHECK_LAUNCH();
   k_sq_inv_x<<<x.B * x.H, kSqThreads, (x.W + m * C) * sizeof(float2), x.st>>>(z, s, twx, x.W, C, m,
-                                                                                scale, hermitian);
+                                                                                scale);
   LBM_CHECK_LAUNCH();
   return LBM_OK;
 }
@@ -1473,28 +1465,28 @@ int sq_forward(const TrCtx& x, const float* params, const float* xin, float* sav
   LBM_CHECK_LAUNCH();
   k_sq_twiddle<<<nb(x.H), 256, 0, x.st>>>(reinterpret_cast<float2*>(x.ws + pl.twy), x.H);
   LBM_CHECK_LAUNCH();
-  LBM_TRY(sq_pw(x, xin, c.c_in + 2, p + o.lift0_w, 0, p + o.lift0_b, nullptr, h, saved + pl.h1pre,
-                ta, 0, 1));
-  LBM_TRY(sq_pw(x, ta, h, p + o.lift1_w, 0, p + o.lift1_b, nullptr, C, nullptr, theta(0), 0, 0));
+  LBM_TRY(sq_pw(x, xin, c.c_in + 2, p + o.lift0_w, p + o.lift0_b, nullptr, h, saved + pl.h1pre,
+                ta, 1));
+  LBM_TRY(sq_pw(x, ta, h, p + o.lift1_w, p + o.lift1_b, nullptr, C, nullptr, theta(0), 0));
   for (int n = 0; n < c.layers; ++n) {
     float2* xh = reinterpret_cast<float2*>(saved + pl.xh) + (size_t)n * spec;
-    LBM_TRY(sq_spectral_fwd(x, theta(n), xh, 0));
+    LBM_TRY(sq_spectral_fwd(x, theta(n), xh));
     k_tr_mix<<<nb(spec), 256, 0, x.st>>>(xh, rt + (size_t)n * 2 * m * m * C * C, yh, B, C, 2 * m * m);
     LBM_CHECK_LAUNCH();
-    LBM_TRY(sq_spectral_inv(x, yh, s, 1.0f / ((float)x.H * (float)x.W), 1));
-    LBM_TRY(sq_pw(x, theta(n), C, p + o.w[n], 0, p + o.b[n], s, C, saved + pl.zpre + (size_t)n * P * C,
-                  theta(n + 1), 0, 1));
+    LBM_TRY(sq_spectral_inv(x, yh, s, 1.0f / ((float)x.H * (float)x.W)));
+    LBM_TRY(sq_pw(x, theta(n), C, p + o.w[n], p + o.b[n], s, C, saved + pl.zpre + (size_t)n * P * C,
+                  theta(n + 1), 1));
   }
   const float* hin = theta(c.layers);
   int fan = C;
   for (int l = 0; l < c.dec_layers; ++l) {
     float* hout = (l % 2 == 0) ? ta : tb;
-    LBM_TRY(sq_pw(x, hin, fan, p + o.dec_w[l], 0, p + o.dec_b[l], nullptr, S,
-                  saved + pl.hdpre + (size_t)l * P * S, hout, 0, 1));
+    LBM_TRY(sq_pw(x, hin, fan, p + o.dec_w[l], p + o.dec_b[l], nullptr, S,
+                  saved + pl.hdpre + (size_t)l * P * S, hout, 1));
     hin = hout;
     fan = S;
   }
-  LBM_TRY(sq_pw(x, hin, fan, p + o.out_w, 0, p + o.out_b, nullptr, c.c_out, nullptr, ycl, 0, 0));
+  LBM_TRY(sq_pw(x, hin, fan, p + o.out_w, p + o.out_b, nullptr, c.c_out, nullptr, ycl, 0));
   k_sq_cl_to_nchw<<<nb(P * c.c_out), 256, 0, x.st>>>(ycl, out_d, B, x.H, x.W, c.c_out);
   LBM_CHECK_LAUNCH();
   return LBM_OK;

@@ -674,11 +674,12 @@ struct StepVariant {
          k_step_tma<TY, ST, MB, kModeMulti>},                                              \
         StepShape<TY, ST, MB>::kSmem, StepShape<TY, ST, MB>::kSmemStats                    \
   }
-static const StepVariant kStepVariants[LBM_STEP_VARIANTS] = {
+static constexpr StepVariant kStepVariants[LBM_STEP_VARIANTS] = {
     LBM_STEP_VARIANT(3, 2, 5), LBM_STEP_VARIANT(4, 2, 4), LBM_STEP_VARIANT(2, 2, 7),
     LBM_STEP_VARIANT(5, 2, 4), LBM_STEP_VARIANT(3, 3, 4), LBM_STEP_VARIANT(6, 2, 3)};
 #undef LBM_STEP_VARIANT
-static_assert(kChunkRows == 4, "the chunk kernels take the tiles of shape kChunkVariant");
+static_assert(kStepVariants[kChunkVariant].ty == kChunkRows,
+              "a chunk kernel has a warp for every row of a tile of shape kChunkVariant");
 
 __global__ void __launch_bounds__(kBlock) k_export(const GridDev* __restrict__ grids, int ngrids,
                                                    const uint32_t* __restrict__ mask,

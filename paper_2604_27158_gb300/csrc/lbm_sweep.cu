@@ -63,8 +63,7 @@ __host__ __device__ constexpr int in_cls(int i) {  // 2 5 6 | 0 1 3 | 4 7 8
   return i == 2 || i == 0 || i == 4 ? 0 : (i == 5 || i == 1 || i == 7 ? 1 : 2);
 }
 
-// cp.async: this lane's own 16 (or 4) bytes, read back by the lane that copied them (and,
-// at a warp's edge columns, by a neighbouring warp of the group after a barrier)
+// cp.async: this lane's own 16 (or 4) bytes, read back by the lane that copied them
 __device__ __forceinline__ void cpa16(uint32_t s, const float* g) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(g) : "memory");
 }
@@ -736,7 +735,6 @@ void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks) {
               const int rw = w + 1 < nw ? w + 1 : (wrap ? 0 : w);
               t.left = (short)(base + lw);
               t.right = (short)(base + rw);
-              t.left_last = (short)std::min(31, end - first - 32 * lw - 1);
             }
             tasks->push_back(t);
           }

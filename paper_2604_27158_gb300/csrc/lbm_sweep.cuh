@@ -19,10 +19,9 @@ struct SweepTask {
   int y0, rows;  // rows == 0: unused slot
   short last;    // last active lane
   short nwarps, bar;  // warps of the group; its named barrier
-  short left, right, left_last;  // neighbouring warps (CTA-relative) and the left one's last lane
-  int pad;
+  short left, right;  // neighbouring warps (CTA-relative)
 };
-static_assert(sizeof(SweepTask) == 40, "task table entry");
+static_assert(sizeof(SweepTask) == 36, "task table entry");
 
 struct Handle;
 // Tasks of a batch, kSweepWarps a CTA.  Host only, a function of the grids alone.
