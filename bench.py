@@ -45,7 +45,7 @@ NX, NY = 512, 256
 TAU, RHO_IN, RHO_OUT = 0.7, 1.001, 1.0
 TOL, CHECK_EVERY = 1e-7, 100
 BYTES_PER_CELL = 72.125  # 9 x 4 B read + 9 x 4 B written + 1 mask bit per cell update
-STEPS_PER_PASS = 2       # lbm_step advances two time steps per pass over the populations
+STEPS_PER_PASS = 2       # time steps of a pass over the populations, where lbm_step takes passes
 REINIT_BYTES_PER_CELL = 56  # (rho, u_x, u_y) read; 9 populations + stored (u_x, u_y) written
 
 
@@ -79,9 +79,10 @@ def parse():
     ap.add_argument("--step-variant", type=int, default=-1,
                     help="step-kernel tile shape index; -1 (default) times all shapes and keeps the fastest")
     ap.add_argument("--case", default=None,
-                    choices=["lbm", "check", "reinit", "fno", "shear_fno"],
+                    choices=["lbm", "single", "check", "reinit", "fno", "shear_fno"],
                     help="run one small case to be profiled and exit (no JSON line): 'lbm' 60 "
-                         "steps of the bench batch (tile shape 3), 'check' 5 steps + 5 "
+                         "steps of the bench batch in two-step passes, 'single' 60 single "
+                         "steps of it (tile shape 3), 'check' 5 steps + 5 "
                          "statistics-only residuals + 5 step+statistics checks of it, "
                          "'reinit' 5 re-initialisations of it from its fields after 20 steps, 'fno' "
                          "8 forwards of the FNO throughput shape, 'shear_fno' 8 forwards of "
@@ -96,13 +97,14 @@ def run_case(args):
     import paper_2604_27158_gb300 as P
     from paper_2604_27158_gb300.fno import Fno, FnoShape
     from paper_2604_27158_gb300.lbm import GridSpec, Lattice
-    if args.case in ("lbm", "check"):
+    if args.case in ("lbm", "single", "check"):
         T = args.trajectories
         masks, _ = workload(T, 0)
         lat = Lattice([GridSpec(NX, NY, TAU, bc_west=P.BC_PRESSURE, bc_east=P.BC_PRESSURE,
                                 west_value=RHO_IN, east_value=RHO_OUT)] * T, masks)
         lat.set_step_variant(3 if args.step_variant < 0 else args.step_variant)
-        if args.case == "lbm":
+        lat.set_passes(args.case == "lbm")
+        if args.case != "check":
             lat.step(60)
         else:
             lat.step(20)
@@ -190,19 +192,53 @@ def read_peaks():
         return 6800.0, "fallback"
 
 
-def step_kernel_traffic(cells, shape):
-    """DRAM bytes per step-kernel launch from the committed ncu record of the tile shape in
-    use, scaled to `cells`; None when there is no record for that shape or the step kernel's
-    source changed since the counters were taken."""
+# The workloads beside the headline one: their lists go to the standard error stream, so that the
+# line on standard output stays short enough (LINE_MAX characters) for readers that keep a tail of it.
+DETAIL_KEYS = ("time_to_steady", "tolerance_ladder", "lbm_sweep", "launch_bound", "hybrid_training",
+               "double_shear", "fno_throughput", "unsteady_hybrid", "autotune_ms")
+LINE_MAX = 2800
+
+
+def rounded(v, digits):
+    """Floats to `digits` significant digits, in any nesting of lists and dicts."""
+    if isinstance(v, float):
+        return float(f"{v:.{digits}g}")
+    if isinstance(v, dict):
+        return {k: rounded(x, digits) for k, x in v.items()}
+    return [rounded(x, digits) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def split_line(line):
+    """(the line for standard output, the details for standard error) of the full record; the line
+    keeps one figure of each workload."""
+    details = {k: v for k, v in line.items() if k in DETAIL_KEYS}
+    short = {k: v for k, v in line.items() if k not in DETAIL_KEYS}
+
+    def figure(key, *path):
+        v = details.get(key)
+        for p in path:
+            v = None if v is None else v[p]
+        return v
+
+    shear, sweep = figure("double_shear", "arms"), details.get("lbm_sweep")
+    short["other"] = {
+        "fno_b32_ms": figure("fno_throughput", "ms_per_forward"),
+        "unsteady_cycle_ms": figure("unsteady_hybrid", "cycle_ms_steady"),
+        "training_step_ms": figure("hybrid_training", "ms_per_step"),
+        "domain_glups": sweep and [d["glups"] for d in sweep],
+        "shear_eps_T": shear and {k: a["eps_T"] for k, a in shear.items() if "eps_T" in a}}
+    return rounded(short, 7), details
+
+
+def pass_kernel_traffic(cells):
+    """DRAM bytes per launch of the two-step pass from the committed ncu record, scaled to `cells`;
+    None when the kernel's source changed since the counters were taken."""
     import hashlib
     try:
-        rec = json.load(open(os.path.join(ROOT, "profiles", "k_step_tma_traffic.json")))
-        src = open(os.path.join(ROOT, "paper_2604_27158_gb300", "csrc", "lbm.cu")).read()
-        a = src.index("// ------------------------------------------------------ the fused step ---")
-        b = src.index("__global__ void __launch_bounds__(kBlock) k_export(")
+        rec = json.load(open(os.path.join(ROOT, "profiles", "k_sweep_traffic.json")))
+        src = open(os.path.join(ROOT, "paper_2604_27158_gb300", "csrc", "lbm_sweep.cu")).read()
+        a, b = src.index("constexpr int kWarps"), src.index("// rcp_lane of n values")
         if hashlib.sha256(src[a:b].encode()).hexdigest()[:16] != rec["source_section_sha256_16"]:
-            return None
-        if rec["variant"] != shape[0]:
             return None
         return rec["traffic_bytes_per_launch"] * cells / rec["cells"]
     except Exception:
@@ -450,6 +486,7 @@ def main():
     else:
         _, tune_ms = lat.autotune(reps=20)
     shape = lat.step_variant()
+    steps_per_launch = STEPS_PER_PASS if lat.passes() else 1
     hyb = Hybrid(lat, net, HybridConfig(use_fno=1, neq_mode=1, check_every=CHECK_EVERY, tol=TOL,
                                         max_steps=args.solve_steps))
     stream = torch.cuda.current_stream()
@@ -488,7 +525,7 @@ def main():
     torch.cuda.synchronize()
     kms = k0.elapsed_time(k1) / nk
     peak, peak_kind = read_peaks()
-    kms *= STEPS_PER_PASS  # of one launch: a pass of two time steps
+    kms *= steps_per_launch  # of one launch
     achieved = BYTES_PER_CELL * cells / (kms * 1e-3) / 1e9
 
     # the re-initialisation kernel (a4) on the same batch, from its macroscopic fields: reads
@@ -651,6 +688,7 @@ def main():
             lat_s = Lattice([gs], [solid])
             _, sw_ms = lat_s.autotune(reps=5)
             sv = lat_s.step_variant()
+            spl = STEPS_PER_PASS if lat_s.passes() else 1
             lat_s.step(200)
             w0, w1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             w0.record(stream)
@@ -664,8 +702,9 @@ def main():
             sweep.append({"nx": sx, "ny": sy, "cells": cells_s, "porosity": fluid_s / cells_s,
                           "f_bytes": 2 * 36 * cells_s, "ms_per_step": sms, "glups": gl,
                           "glups_fluid_only": fluid_s / (sms * 1e-3) / 1e9,
-                          "frac_of_measured_hbm": gl * BYTES_PER_CELL / STEPS_PER_PASS / peak,
-                          "frac_of_8tbs": gl * BYTES_PER_CELL / STEPS_PER_PASS / 8000.0,
+                          "frac_of_measured_hbm": gl * BYTES_PER_CELL / spl / peak,
+                          "frac_of_8tbs": gl * BYTES_PER_CELL / spl / 8000.0,
+                          "steps_per_launch": spl,
                           "tile_shape": {"rows_per_tile": sv[1], "stages": sv[2],
                                          "ctas_per_sm": sv[3]}})
             lat_s.close()
@@ -1050,12 +1089,12 @@ def main():
             "config": bench_config(T, phis, args.solve_steps, world),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "peak_kind": peak_kind,
-                         "kernel": "k_sweep", "bytes_per_launch": BYTES_PER_CELL * cells,
-                         "steps_per_launch": STEPS_PER_PASS,
+                         "kernel": "k_sweep" if steps_per_launch > 1 else "k_step_tma",
+                         "bytes_per_launch": BYTES_PER_CELL * cells,
+                         "steps_per_launch": steps_per_launch,
                          "check_step_tile_shape": {"rows_per_tile": shape[1], "stages": shape[2],
-                                        "ctas_per_sm": shape[3], "autotune_ms": tune_ms},
-                         "launch_ms": kms,
-                         "single_step_kernel_traffic": step_kernel_traffic(cells, shape),
+                                                   "ctas_per_sm": shape[3]},
+                         "launch_ms": kms, "traffic": pass_kernel_traffic(cells) if steps_per_launch > 1 else None,
                          "traffic_unit": "bytes per launch (ncu dram read + write)"},
             "reinit_kernel": reinit_kernel,
             "time_to_steady_summary": None if tts is None else {
@@ -1075,6 +1114,7 @@ def main():
             "double_shear": shear,
             "fno_throughput": fno_tp,
             "unsteady_hybrid": unsteady,
+            "autotune_ms": tune_ms,
             "gpu_launches": None,
             "clocks": clk.summary(),
             "e2e": e2e,
@@ -1090,10 +1130,13 @@ def main():
         lbm_k, done = 0, 0
         for c in range(checks):  # a check's step opens the next interval
             n = min(CHECK_EVERY, steps_per_solve - done) - (1 if c else 0)
-            lbm_k += n - n // 4 * 4 // STEPS_PER_PASS  # four steps at a time are two passes
+            # four steps at a time are two passes
+            lbm_k += n - (n // 4 * 4 // STEPS_PER_PASS if steps_per_launch > 1 else 0)
             done = min(done + CHECK_EVERY, steps_per_solve)
         per_step = fno_k + 1 + 1 + 2 + lbm_k + 3 * checks
         line["gpu_launches"] = per_step * args.steps
+        line, details = split_line(line)
+        print("details " + json.dumps(details), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     hyb.close()
     lat.close()
