@@ -467,15 +467,17 @@ __global__ void __launch_bounds__(kLiftThreads, lift_ctas_per_sm(kCin, kC))
 // hidden layers, other widths); FP32 throughout.  A thread owns kNP pixels of the output grid (the
 // padded grid is cropped): its hidden units stay in registers, packed over pairs of inputs, and
 // every 16-byte broadcast load of weights from shared memory feeds 2 kNP packed multiply-adds, which
-// bound it.  Widths below kS are padded with zero weights.  (Hidden units in indexed arrays, as
-// they were, live in local memory: three layers of 32 on 256 x 512 pixels took 110 us.)
+// bound it.  Inputs of a layer are padded to kS (8, 16, 32 or 64) with zero weights, its outputs to
+// whole fours.  (Hidden units in indexed arrays, as they were, live in local memory: three layers of
+// 32 on 256 x 512 pixels took 110 us.  Padded to 32 at least, a forward with eight layers of 1 to 8
+// units on 8 x 256^2 pixels took 330 us, with the indexed arrays 74 to 162, so 77 to 90.)
 // The layer loop stays rolled: four outputs at a time go to the thread's own column of shared
 // memory (conflict-free) and are read back as the next layer's inputs.
-template <int kF2, int kNP>
-__device__ __forceinline__ void dec_layer(const float* w, const float* bias, int S, int act,
+template <int kS, int kF2, int kNP>
+__device__ __forceinline__ void dec_layer(const float* w, const float* bias, int outs, int act,
                                           const float2 (*in)[kF2], float* col) {
 #pragma unroll 1
-  for (int j = 0; j < S; j += 4) {
+  for (int j = 0; j < outs; j += 4) {
     float2 acc[kNP][4];
 #pragma unroll
     for (int q = 0; q < kNP; ++q)
@@ -505,7 +507,7 @@ __device__ __forceinline__ void dec_layer(const float* w, const float* bias, int
         v0 = make_float2(act_tc(v0.x, act), act_tc(v0.y, act));
         v1 = make_float2(act_tc(v1.x, act), act_tc(v1.y, act));
       }
-      float* o = col + (q * S + j) * 128;
+      float* o = col + (q * kS + j) * 128;
       o[0] = v0.x;
       o[128] = v0.y;
       o[256] = v1.x;
@@ -513,6 +515,7 @@ __device__ __forceinline__ void dec_layer(const float* w, const float* bias, int
     }
   }
 }
+__host__ __device__ constexpr int dec_out_pad(int S) { return S < 16 ? 16 : S; }
 template <int kC, int kS, int kNP>
 __global__ void __launch_bounds__(128)
     k_decoder_deep(const __nv_bfloat16* __restrict__ theta, float* __restrict__ out,
@@ -520,7 +523,8 @@ __global__ void __launch_bounds__(128)
                    int nlayers, int B, TcGrid gd, int S, int cout, int act) {
   extern __shared__ __align__(16) float dec_s[];
   pdl_trigger();
-  // layout: w of layer 0 [kS][kC], of the others [kS][kS], out.w [cout][kS]; their biases [kS]
+  // layout: w of layer 0 [kS][kC], of the others [kS][kS], out.w [cout][kS]; their biases [kS], the
+  // outputs' (up to 16) [dec_out_pad(kS)]
   float* const bias_s = dec_s + kS * kC + (nlayers - 1) * kS * kS + cout * kS;
   for (int l = 0, at = 0, fan = kC; l <= nlayers; ++l) {
     const int rows = l < nlayers ? kS : cout, have = l < nlayers ? S : cout;
@@ -559,7 +563,7 @@ __global__ void __launch_bounds__(128)
       for (int u = 0; u < 4; ++u) a[q][g * 4 + u] = __bfloat1622float2(hv[u]);
     }
   }
-  float* const col = bias_s + (nlayers + 1) * kS + threadIdx.x;  // [kNP][kS][128]
+  float* const col = bias_s + nlayers * kS + dec_out_pad(kS) + threadIdx.x;  // [kNP][kS][128]
   auto reload = [&]() {
 #pragma unroll
     for (int q = 0; q < kNP; ++q)
@@ -567,12 +571,16 @@ __global__ void __launch_bounds__(128)
       for (int c = 0; c < kS / 2; ++c)
         h[q][c] = make_float2(col[(q * kS + 2 * c) * 128], col[(q * kS + 2 * c + 1) * 128]);
   };
-  dec_layer<kC / 2, kNP>(dec_s, bias_s, kS, act, a, col);
+  const int outs = (S + 3) & ~3;
+  for (int j = outs; j < kS; ++j)  // columns that no layer writes
+#pragma unroll
+    for (int q = 0; q < kNP; ++q) col[(q * kS + j) * 128] = 0.0f;
+  dec_layer<kS, kC / 2, kNP>(dec_s, bias_s, outs, act, a, col);
   reload();
   const float* w = dec_s + kS * kC;
 #pragma unroll 1
   for (int l = 1; l < nlayers; ++l, w += kS * kS) {
-    dec_layer<kS / 2, kNP>(w, bias_s + l * kS, kS, act, h, col);
+    dec_layer<kS, kS / 2, kNP>(w, bias_s + l * kS, outs, act, h, col);
     reload();
   }
 #pragma unroll 1
@@ -1799,19 +1807,20 @@ static int fno_forward_tc_impl(const fno_config& c, const FnoTcParams& P, const 
       LBM_TRY(launch_pdl((k_decoder_tc<kC, 64, kAct>), dim3(ctas), dim3(kDecThreads), smem_tc, s,
                          th[cur], out, P.params, P.dec_offs, B, gd, c.c_out, status));
   } else {
-    const int S = c.dec_size <= 32 ? 32 : 64, np = S == 32 ? 2 : 1;
+    const int S = c.dec_size <= 8 ? 8 : (c.dec_size <= 16 ? 16 : (c.dec_size <= 32 ? 32 : 64));
+    const int np = S <= 32 ? 2 : 1;
     const size_t dec_smem =
         ((size_t)S * kC + (size_t)(c.dec_layers - 1) * S * S + (size_t)c.c_out * S +
-         (size_t)(c.dec_layers + 1) * S + (size_t)np * S * 128) * sizeof(float);
+         (size_t)c.dec_layers * S + dec_out_pad(S) + (size_t)np * S * 128) * sizeof(float);
     const dim3 blocks((unsigned)((pix + 128 * np - 1) / (128 * np)));
-    if (S == 32)
-      LBM_TRY(launch_pdl((k_decoder_deep<kC, 32, 2>), blocks, dim3(128), dec_smem, s, th[cur], out,
-                         P.params, P.dec_offs, c.dec_layers, B, gd, c.dec_size, c.c_out,
-                         c.activation));
-    else
-      LBM_TRY(launch_pdl((k_decoder_deep<kC, 64, 1>), blocks, dim3(128), dec_smem, s, th[cur], out,
-                         P.params, P.dec_offs, c.dec_layers, B, gd, c.dec_size, c.c_out,
-                         c.activation));
+    auto run = [&](auto kernel) {
+      return launch_pdl(kernel, blocks, dim3(128), dec_smem, s, th[cur], out, P.params, P.dec_offs,
+                        c.dec_layers, B, gd, c.dec_size, c.c_out, c.activation);
+    };
+    LBM_TRY(S == 8    ? run(k_decoder_deep<kC, 8, 2>)
+            : S == 16 ? run(k_decoder_deep<kC, 16, 2>)
+            : S == 32 ? run(k_decoder_deep<kC, 32, 2>)
+                      : run(k_decoder_deep<kC, 64, 1>));
   }
   return LBM_OK;
 }
@@ -1853,6 +1862,10 @@ static int tc_set_smem_attrs() {
   if constexpr (kC <= 32)
     LBM_CHECK_CUDA(cudaFuncSetAttribute(k_mix4<kC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         kTcSmemMax));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_decoder_deep<kC, 8, 2>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemMax));
+  LBM_CHECK_CUDA(cudaFuncSetAttribute(k_decoder_deep<kC, 16, 2>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemMax));
   LBM_CHECK_CUDA(cudaFuncSetAttribute(k_decoder_deep<kC, 32, 2>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemMax));
   LBM_CHECK_CUDA(cudaFuncSetAttribute(k_decoder_deep<kC, 64, 1>,
