@@ -42,6 +42,7 @@ constexpr int kDftX = 32;        // columns of one of its stages
 constexpr int kDftYA = 8;        // kept rows of a forward y-DFT thread
 constexpr int kDftYC = 64;       // rows of one of its stages
 constexpr int kInvY = 8;         // rows of an inverse y-DFT thread
+__host__ __device__ constexpr int y_chunks(int mc) { return (mc + 63) / 64; }  // blocks of an item's m C columns
 
 struct TrOff {
   size_t lift0_w, lift0_b, lift1_w, lift1_b;
@@ -809,17 +810,22 @@ __global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f
 
 // Forward y-DFT over the kept rows: Xh[b][a][kx][c] = scale(kx) sum_y X1[b][y][kx][c]
 // e^{-2 pi i ky(a) y / H}, ky(a) = a (a < m) or H - 2m + a; scale = 1, or c_kx / (H W)
-// for the adjoint of the real inverse transform.  A block takes one (b, kx) and kDftYA kept
-// rows; a lane two channels, a warp every eighth y; the warps' sums are added in order.
+// for the adjoint of the real inverse transform.  A block takes 32 pairs of a batch item's m C
+// columns (kx, c), a lane one pair, and kDftYA kept rows; a warp every eighth y; the warps' sums
+// are added in order.  (With one kx a block, networks of 8 channels used four lanes of a warp and
+// the same table rows in eight blocks: 32 items of 64 x 58, 29 modes, took 1.66 ms a training pass,
+// now 0.91.)
 __global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
                                                   float2* __restrict__ xh,
                                                   const float4* __restrict__ ey, int H, int W,
                                                   int C, int m, int adjoint_scale, int vec) {
   __shared__ float4 es[kDftYC][kDftYA];
   __shared__ float4 red[kDftYA][32];
-  const int b = blockIdx.x / m, kx = blockIdx.x % m, a0 = blockIdx.y * kDftYA;
+  const int mc = m * C, nch = y_chunks(mc);
+  const int b = blockIdx.x / nch, a0 = blockIdx.y * kDftYA;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const bool on = 2 * lane < C;
+  const int at = 2 * (32 * (int)(blockIdx.x % nch) + lane);  // the lane's first column
+  const bool on = at < mc;
   float2 acc[kDftYA][2];
 #pragma unroll
   for (int a = 0; a < kDftYA; ++a) acc[a][0] = acc[a][1] = make_float2(0.0f, 0.0f);
@@ -836,7 +842,7 @@ __global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
 #pragma unroll 4
       for (int y = wp; y < n; y += 8) {
         const float4 v = *reinterpret_cast<const float4*>(
-            x1 + (((size_t)b * H + y0 + y) * m + kx) * C + 2 * lane);
+            x1 + ((size_t)b * H + y0 + y) * mc + at);
 #pragma unroll
         for (int a = 0; a < kDftYA; ++a) {
           const float4 e = es[y][a];
@@ -859,11 +865,11 @@ __global__ void __launch_bounds__(256) k_tr_dft_y(const float2* __restrict__ x1,
     }
     __syncthreads();
   }
-  const float sc = adjoint_scale ? (kx == 0 ? 1.0f : 2.0f) / ((float)H * (float)W) : 1.0f;
+  const float sc = adjoint_scale ? (at < C ? 1.0f : 2.0f) / ((float)H * (float)W) : 1.0f;
   const int a = wp;  // kDftYA == 8 warps
   if (on && a0 + a < 2 * m) {
     const float4 r = red[a][lane];
-    float2* o = xh + (((size_t)b * 2 * m + a0 + a) * m + kx) * C + 2 * lane;
+    float2* o = xh + ((size_t)b * 2 * m + a0 + a) * mc + at;
     if (vec) {
       *reinterpret_cast<float4*>(o) = make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sc);
     } else {
@@ -1176,7 +1182,7 @@ __global__ void k_tr_mix_bwd_r(const float2* __restrict__ xh, const float2* __re
 
 // Inverse y-DFT: Z[b][y][kx][c] = w(kx) scale sum_a Yh[b][a][kx][c] e^{+2 pi i ky(a) y / H},
 // w(kx) = c_kx (forward) or 1 (adjoint of the forward DFT), ready for the pointwise kernel.  A
-// block takes one (b, kx) and 8 warps x kInvY rows; a lane two channels.
+// block takes 32 pairs of an item's columns (kx, c), as k_tr_dft_y, and 8 warps x kInvY rows.
 __global__ void __launch_bounds__(256) k_tr_inv_y(const float2* __restrict__ yh,
                                                   float2* __restrict__ z,
                                                   const float4* __restrict__ ey, int H, int C,
@@ -1185,17 +1191,19 @@ __global__ void __launch_bounds__(256) k_tr_inv_y(const float2* __restrict__ yh,
   constexpr int YB = 8 * kInvY, EP = YB + 1;
   float4* es = reinterpret_cast<float4*>(sm);       // [2m][EP]
   float4* col = es + 2 * m * EP;                    // [2m][32]
-  const int b = blockIdx.x / m, kx = blockIdx.x % m, y0 = blockIdx.y * YB;
+  const int mc = m * C, nch = y_chunks(mc);
+  const int b = blockIdx.x / nch, y0 = blockIdx.y * YB;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const bool on = 2 * lane < C;
+  const int at0 = 64 * (int)(blockIdx.x % nch), at = at0 + 2 * lane;  // first columns: block, lane
+  const bool on = at < mc;
   for (int j = threadIdx.x; j < 2 * m * YB; j += 256) {
     const int y = j / (2 * m), a = j - y * (2 * m);
     es[a * EP + y] = y0 + y < H ? ey[(size_t)(y0 + y) * 2 * m + a] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   for (int j = threadIdx.x; j < 2 * m * 32; j += 256) {
     const int a = j >> 5, l = j & 31;
-    if (2 * l < C)
-      col[j] = *reinterpret_cast<const float4*>(yh + (((size_t)b * 2 * m + a) * m + kx) * C + 2 * l);
+    if (at0 + 2 * l < mc)
+      col[j] = *reinterpret_cast<const float4*>(yh + ((size_t)b * 2 * m + a) * mc + at0 + 2 * l);
   }
   __syncthreads();
   if (!on) return;
@@ -1214,12 +1222,12 @@ __global__ void __launch_bounds__(256) k_tr_inv_y(const float2* __restrict__ yh,
       acc[y][1] = __ffma2_rn(dup2(v.w), make_float2(e.y, e.w), acc[y][1]);
     }
   }
-  const float w = (hermitian && kx > 0) ? 2.0f * scale : scale;
+  const float w = (hermitian && at >= C) ? 2.0f * scale : scale;
 #pragma unroll
   for (int y = 0; y < kInvY; ++y) {
     const int yy = y0 + wp * kInvY + y;
     if (yy < H)
-      *reinterpret_cast<float4*>(z + (((size_t)b * H + yy) * m + kx) * C + 2 * lane) =
+      *reinterpret_cast<float4*>(z + ((size_t)b * H + yy) * mc + at) =
           make_float4(acc[y][0].x * w, acc[y][0].y * w, acc[y][1].x * w, acc[y][1].y * w);
   }
 }
@@ -1383,7 +1391,7 @@ int spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_scale)
       f, x1, reinterpret_cast<const float*>(x.ws + x.pl.ex), rows, x.W, C, cp, m, ng, ks, ep,
       vec_of(f, C));
   LBM_CHECK_LAUNCH();
-  k_tr_dft_y<<<dim3(x.B * m, nb(2 * m, kDftYA)), 256, 0, x.st>>>(
+  k_tr_dft_y<<<dim3(x.B * y_chunks(m * C), nb(2 * m, kDftYA)), 256, 0, x.st>>>(
       x1, out, reinterpret_cast<const float4*>(x.ws + x.pl.ey), x.H, x.W, C, m, adjoint_scale,
       vec_of(out, 4));
   LBM_CHECK_LAUNCH();
@@ -1395,7 +1403,7 @@ int spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_scale)
 size_t inv_y_smem(int m) { return sizeof(float4) * 2 * m * (8 * kInvY + 1 + 32); }
 int spectral_inv(const TrCtx& x, const float2* coef, float scale, int hermitian) {
   const int C = x.c->width, m = x.c->modes;
-  k_tr_inv_y<<<dim3(x.B * m, nb(x.H, 8 * kInvY)), 256, inv_y_smem(m), x.st>>>(
+  k_tr_inv_y<<<dim3(x.B * y_chunks(m * C), nb(x.H, 8 * kInvY)), 256, inv_y_smem(m), x.st>>>(
       coef, reinterpret_cast<float2*>(x.ws + x.pl.z),
       reinterpret_cast<const float4*>(x.ws + x.pl.ey), x.H, C, m, scale, hermitian);
   LBM_CHECK_LAUNCH();
