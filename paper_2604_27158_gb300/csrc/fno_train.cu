@@ -722,17 +722,19 @@ __global__ void __launch_bounds__(256) k_tr_wgrad_reduce(const float* __restrict
 // frequencies (accumulators (Re, Im) packed) of every ks-th column; the column slices are
 // added in order.  Bound by FP32 multiply-adds and the one read of f; stages are double
 // buffered.
+// Where its blocks leave multiprocessors idle it takes fewer rows, and 16 warps instead of 8, that is
+// more and shorter column slices: its time is then one block's.  (Eight channels, 29 modes, one item
+// of 100 x 1000, a training pass: 1.00 -> 0.71 ms.)
 template <int NP>
-__global__ void __launch_bounds__(256, 2) k_tr_dft_x(const float* __restrict__ f,
+__global__ void __launch_bounds__(512, 1) k_tr_dft_x(const float* __restrict__ f,
                                                      float2* __restrict__ x1,
                                                      const float* __restrict__ ex, size_t rows,
-                                                     int W, int C, int cp, int m, int ng, int ks,
-                                                     int ep, int vec) {
+                                                     int W, int C, int cp, int rpb, int m, int ng,
+                                                     int ks, int ep, int vec) {
   extern __shared__ __align__(16) float sm[];
   const int stage = kDftX * (kDftM + ep);
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int kg = wp % ng, sl = wp / ng;
-  const int rpb = kDftM / cp;
   const size_t row0 = (size_t)blockIdx.x * rpb;
   const int nr = (int)min((size_t)rpb, rows - row0);
   const int nthr = blockDim.x;
@@ -1383,12 +1385,14 @@ int spectral_fwd(const TrCtx& x, const float* f, float2* out, int adjoint_scale)
   const int C = x.c->width, m = x.c->modes, np = x.pl.np, ng = x.pl.ng, ep = x.pl.ep;
   float2* x1 = reinterpret_cast<float2*>(x.ws + x.pl.x1);
   const int cp = C <= 8 ? 8 : (C <= 16 ? 16 : (C <= 32 ? 32 : 64));
-  const int ks = std::max(1, 8 / ng);
   const size_t rows = (size_t)x.B * x.H;
+  int rpb = kDftM / cp;  // rows a block
+  const int ks = std::max(1, (nb(rows, rpb) < (unsigned)kTrSms ? 16 : 8) / ng);
+  while (rpb > 1 && nb(rows, rpb) < (unsigned)kTrSms) rpb /= 2;
   auto kernel = np == 4 ? k_tr_dft_x<4> : (np == 6 ? k_tr_dft_x<6> : (np == 7 ? k_tr_dft_x<7>
                                                                               : k_tr_dft_x<8>));
-  kernel<<<nb(rows, kDftM / cp), 32 * ng * ks, dft_x_smem(ep, np, ng), x.st>>>(
-      f, x1, reinterpret_cast<const float*>(x.ws + x.pl.ex), rows, x.W, C, cp, m, ng, ks, ep,
+  kernel<<<nb(rows, rpb), 32 * ng * ks, dft_x_smem(ep, np, ng), x.st>>>(
+      f, x1, reinterpret_cast<const float*>(x.ws + x.pl.ex), rows, x.W, C, cp, rpb, m, ng, ks, ep,
       vec_of(f, C));
   LBM_CHECK_LAUNCH();
   k_tr_dft_y<<<dim3(x.B * y_chunks(m * C), nb(2 * m, kDftYA)), 256, 0, x.st>>>(
