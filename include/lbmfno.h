@@ -233,9 +233,10 @@ int lbm_stream_probe(lbm_handle* h, int variant, void* stream);
  * this batch (reading the current state, writing only the scratch buffer: the state is
  * unchanged), selects the fastest, and optionally returns the per-shape milliseconds per
  * step (ms_h, LBM_STEP_VARIANTS entries, INFINITY for shapes that do not fit) and the
- * chosen index.  It then times two single steps of that shape against one pass over two
- * steps, and lbm_step takes passes if they are faster (before: if the estimate of
- * lbm_query_passes says so).  Synchronises `stream`.
+ * chosen index.  Unless passes over two steps are estimated to be faster by 20% or more, it
+ * then times two single steps of that shape against one pass, and lbm_step takes passes if
+ * they are faster (before: if the estimate of lbm_query_passes says so).  Synchronises
+ * `stream`.
  */
 #define LBM_STEP_VARIANTS 6
 int lbm_autotune(lbm_handle* h, int reps, float* ms_h, int* chosen_h, void* stream);

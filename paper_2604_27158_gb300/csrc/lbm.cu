@@ -922,7 +922,7 @@ __global__ void __launch_bounds__(32 * kChunkRows) k_vorticity_chunk(
 struct WsPlan {
   size_t grids_off, uprev_off, seg_off, partial_off, stats_off, status_off, bar_off, tiles_off,
       sweep_off, total;
-  bool passes;  // what sweep_pays estimates
+  double gain;  // what sweep_gain estimates
 };
 
 // Scratch of one statistics evaluation: FP32 row-segment partials, FP64 block sums,
@@ -1038,7 +1038,7 @@ static int plan_layout(const lbm_grid* grids, int ngrids, lbm_layout* lay,
       n += (size_t)d.nseg * ((d.ny + kStepVariants[v].ty - 1) / kStepVariants[v].ty);
     one_wave = one_wave || n <= (size_t)kSweepSms * kStepVariants[v].minb;
   }
-  w.passes = sweep_pays(all, sweep, one_wave);
+  w.gain = sweep_gain(all, sweep, one_wave);
   lay->f_elems = (size_t)kQ * plane_all;
   lay->mask_words = words;
   lay->cells = cells;
@@ -1187,7 +1187,7 @@ int lbm_query_passes(const lbm_grid* grids_h, int ngrids, int* on_h) {
   lbm_layout lay;
   WsPlan wp;
   LBM_TRY(plan_layout(grids_h, ngrids, &lay, nullptr, &wp));
-  *on_h = wp.passes;
+  *on_h = wp.gain >= kSweepGain;
   return LBM_OK;
 }
 
@@ -1243,7 +1243,8 @@ int lbm_init(const lbm_grid* grids_h, int ngrids, const uint32_t* mask_d, float*
   sweep_plan(h->gd, &sweep);
   h->sweep_d = reinterpret_cast<SweepTask*>(ws + wp.sweep_off);
   h->sweep_ctas = (int)(sweep.size() / kSweepWarps);
-  h->sweep = wp.passes;
+  h->sweep_gain = wp.gain;
+  h->sweep = wp.gain >= kSweepGain;
   h->stats_h.assign((size_t)ngrids * R_COUNT, 0.0);
   h->u_max2 = (float)(u_max * u_max);
   cudaStream_t s = S(stream);
@@ -1480,11 +1481,11 @@ int lbm_autotune(lbm_handle* h, int reps, float* ms_h, int* chosen_h, void* stre
       best = v;
     }
   }
-  // two steps of that shape against one pass, in turn, the better of two runs each; enough launches
-  // that a run of short ones takes some 0.1 ms
+  // two steps of that shape against one pass (unless the estimate leaves no doubt), in turn, the
+  // better of two runs each; enough launches that a run of short ones takes some 0.1 ms
   float two_ms[2] = {INFINITY, INFINITY};
   const int n = rc == LBM_OK ? std::max(reps, std::min(16, (int)(0.1f / best_ms))) : 0;
-  for (int k = 0; k < 4 && rc == LBM_OK; ++k) {
+  for (int k = 0; k < 4 && rc == LBM_OK && h->sweep_gain < kSweepSure; ++k) {
     const bool pass = k & 1;
     auto launch = [&] {
       return pass ? sweep_launch(h, src, scratch, s) : launch_step(h, best, kModeStep, src, scratch, s);
@@ -1507,7 +1508,10 @@ int lbm_autotune(lbm_handle* h, int reps, float* ms_h, int* chosen_h, void* stre
   }
   h->variant = best;
   // within 4% the setting stays (these launches read one clean buffer again and again)
-  if (fabsf(two_ms[1] - two_ms[0]) > 0.04f * two_ms[0]) h->sweep = two_ms[1] < two_ms[0];
+  if (h->sweep_gain >= kSweepSure)
+    h->sweep = true;
+  else if (fabsf(two_ms[1] - two_ms[0]) > 0.04f * two_ms[0])
+    h->sweep = two_ms[1] < two_ms[0];
   if (chosen_h) *chosen_h = best;
   return LBM_OK;
 }

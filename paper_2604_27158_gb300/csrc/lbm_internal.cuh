@@ -28,6 +28,7 @@ struct Handle {
   struct SweepTask* sweep_d = nullptr;  // tasks of a multi-step pass (workspace)
   int sweep_ctas = 0;
   bool sweep = false;  // lbm_step takes passes where it may
+  double sweep_gain = 0.0;  // their estimated gain
   unsigned* status_d = nullptr;
   unsigned status_h = 0;
   const uint32_t* mask = nullptr;

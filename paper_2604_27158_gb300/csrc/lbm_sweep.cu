@@ -25,7 +25,7 @@
 // those of single steps.
 //
 // What bounds it (64 grids of 512 x 256): 57 us a step.  The pass moves 5.3 TB/s; issue
-// slots are 46% busy with the eleven warps a multiprocessor that the shared memory of the
+// slots are 47% busy with the eleven to twelve warps a multiprocessor that the shared memory of the
 // kept rows allows, and their fixed-latency chains are what is left.  Measured and not kept:
 // two cells a lane and 24 warps (89 us: the per-lane work is not halved), the kept rows in
 // registers (79 us with 8 warps, or spills), three steps a pass (132 us: 8 warps).
@@ -758,10 +758,12 @@ void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks) {
 // So passes lose where rows are just too many for one wave of one-row tasks and a single step is
 // still one wave (eight forced grids of 180 x 119: 6.4 us a step, 7.2 in passes; 20 grids of 122 x
 // 120: 7.3 and 9.3), and on many narrow or ragged rows.  Taken from an estimated gain of 4% on.
-// Of 500 other batches 439 take passes then, 10 of them at less than 0.98 of the speed of single
-// steps (0.91 the least), and 11 of the other 61 would gain more than 10%.  After lbm_autotune,
-// which times both, 457 take passes, 3 at less than 0.98 (0.96), and none would gain 2%.
-bool sweep_pays(const std::vector<GridDev>& gd, const std::vector<SweepTask>& tasks, bool one_wave) {
+// Of 1,000 other batches 879 take passes then, 12 of them at less than 0.98 of the speed of single
+// steps (0.91 the least), and 24 of the other 121 would gain more than 10%.  After lbm_autotune,
+// which times both, 918 take passes, 6 at less than 0.98 (0.97), and 2 of the others would gain more
+// than 2% (8%).  It takes an estimate of 1.2 or more as it is: of 845 such batches the least gain
+// was 1.02.
+double sweep_gain(const std::vector<GridDev>& gd, const std::vector<SweepTask>& tasks, bool one_wave) {
   double cells = 0, segs = 0, forced = 0, ragged = 0, open = 0, narrow = 0;
   for (const GridDev& d : gd) {
     const double c = (double)d.nx * d.ny;
@@ -787,7 +789,7 @@ bool sweep_pays(const std::vector<GridDev>& gd, const std::vector<SweepTask>& ta
   const double kind = 0.86 * ragged + 0.44 * open + 0.41 * narrow;
   auto iteration = [&](int k) { return base[k] + force[k] * forced + kind; };
   const double pass = 1.56 + (rows + 2) * (full * iteration(kCtas) + iteration(last));
-  return kSweepSteps * step >= 1.04 * pass;
+  return kSweepSteps * step / pass;
 }
 
 int sweep_init() {

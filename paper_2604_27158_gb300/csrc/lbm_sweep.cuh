@@ -26,9 +26,11 @@ static_assert(sizeof(SweepTask) == 36, "task table entry");
 struct Handle;
 // Tasks of a batch, kSweepWarps a CTA.  Host only, a function of the grids alone.
 void sweep_plan(const std::vector<GridDev>& gd, std::vector<SweepTask>* tasks);
-// Whether passes of these tasks are estimated to beat single steps; one_wave: a single step's tiles
-// are resident at once in some shape.  Host only.
-bool sweep_pays(const std::vector<GridDev>& gd, const std::vector<SweepTask>& tasks, bool one_wave);
+// Estimated time of two single steps over that of a pass of these tasks; one_wave: a single step's
+// tiles are resident at once in some shape.  Host only.
+constexpr double kSweepGain = 1.04;  // from here on lbm_step takes passes
+constexpr double kSweepSure = 1.2;   // ... and lbm_autotune does not measure
+double sweep_gain(const std::vector<GridDev>& gd, const std::vector<SweepTask>& tasks, bool one_wave);
 int sweep_init();
 int sweep_launch(Handle* h, const float* src, float* dst, cudaStream_t s);
 
